@@ -103,6 +103,24 @@ __device__ __forceinline__ GridView sub_grid(const GridView &g, int k) {
     return s;
 }
 
+// ------------------------------------------------------------------ packed FP32 pairs
+// Two FP32 values in a 64-bit register pair.  fma.rn.f32x2 rounds each half as fmaf does, so a sum formed
+// with it equals the scalar one bit for bit at half the instructions.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 f2_pack(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(f32x2 v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
 // ------------------------------------------------------------------ activations
 __device__ __forceinline__ float softplus_f32(float s, float beta, float inv_beta) {
     // max(s, 0) + log(1 + exp(-beta |s|)) / beta

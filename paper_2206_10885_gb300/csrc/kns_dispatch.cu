@@ -19,9 +19,15 @@ static cudaError_t dispatch(const Shape &sh, F &&f) {
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_sdf_f32(const Shape &sh, const GridView &g, const float *pts, int64_t n, float *sdf,
-                           float *feat, float *grad, cudaStream_t s) {
-    return dispatch(sh, [&](auto c) { return launch_sdf_cfg<decltype(c)>(g, pts, n, sdf, feat, grad, s); });
+cudaError_t launch_points_direct(const Shape &sh, const GridView &g, const float *pts, int64_t n, float *sdf,
+                                 float *feat, float *grad, cudaStream_t s) {
+    return dispatch(sh, [&](auto c) { return launch_points_direct_cfg<decltype(c)>(g, pts, n, sdf, feat, grad, s); });
+}
+cudaError_t launch_points_tiles(const Shape &sh, const GridView &g, const PointsScratch &sc, int64_t n, float *sdf,
+                                float *feat, float *grad, int sm_count, cudaStream_t s) {
+    return dispatch(sh, [&](auto c) {
+        return launch_points_tiles_cfg<decltype(c)>(g, sc, n, sdf, feat, grad, sm_count, s);
+    });
 }
 
 cudaError_t launch_occupancy_f32(const Shape &sh, const GridView &g, float thresh, uint32_t *words,

@@ -1,31 +1,9 @@
-// kns_fp32.cu -- FP32 CUDA-core kernels: batch field query (Sec. 3.3's per-cell MLP query) and the
-// occupancy-mask build.  One thread per point / voxel; the per-thread MLP evaluators live in
-// kns_device.cuh.
+// kns_fp32.cu -- FP32 CUDA-core kernels with one thread per voxel or ray: the occupancy-mask build and the
+// FP32 refinement of BF16 renders.  The per-thread MLP evaluators live in kns_device.cuh.
 // kns:instantiate (compiled once per grid configuration)
 #include "kns_wave.cuh"
 
 namespace kns {
-
-// Batch field query: d, z and grad d of cell m(x) at each point.
-template <class C>
-__global__ void __launch_bounds__(128) sdf_batch_kernel(GridView g, const float *__restrict__ pts, int64_t n,
-                                                        float *sdf, float *feat, float *grad) {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    const float x = pts[3 * q], y = pts[3 * q + 1], z = pts[3 * q + 2];
-    const int cell = cell_of(g, x, y, z);
-    const float *cw = g.w + (int64_t)cell * g.cell_stride;
-    float zf[FEAT], gr[3];
-    const float d = sdf_full_f32<C>(cw, x, y, z, g.beta, g.inv_beta, zf, gr);
-    sdf[q] = d;
-    if (feat)
-        for (int k = 0; k < FEAT; ++k) feat[q * FEAT + k] = zf[k];
-    if (grad) {
-        grad[3 * q] = gr[0];
-        grad[3 * q + 1] = gr[1];
-        grad[3 * q + 2] = gr[2];
-    }
-}
 
 // Occupancy: voxel v is occupied iff |d(centre of v)| < thresh; the voxel's cell is exact
 // (voxels nest inside cells).  One thread per voxel, x fastest; a warp writes one 32-bit word.
@@ -125,13 +103,6 @@ cudaError_t launch_refine_cfg(const GridView &g, const WaveArgs &a, int sm_count
     return cudaGetLastError();
 }
 template <class C>
-cudaError_t launch_sdf_cfg(const GridView &g, const float *pts, int64_t n, float *sdf, float *feat, float *grad,
-                           cudaStream_t s) {
-    const int64_t blocks = (n + 127) / 128;
-    sdf_batch_kernel<C><<<(unsigned)blocks, 128, 0, s>>>(g, pts, n, sdf, feat, grad);
-    return cudaGetLastError();
-}
-template <class C>
 cudaError_t launch_occ_cfg(const GridView &g, float thresh, uint32_t *words, cudaStream_t s) {
     const int64_t nvox = (int64_t)g.occ_res * g.occ_res * g.occ_res;
     occupancy_kernel<C><<<(unsigned)((nvox + 127) / 128), 128, 0, s>>>(g, thresh, words);
@@ -141,8 +112,6 @@ cudaError_t launch_occ_cfg(const GridView &g, float thresh, uint32_t *words, cud
 // One object file per grid configuration: the build compiles this file once per (W, H, L, LD).
 #ifdef KNS_W
 using InstCfg = Cfg<KNS_W, KNS_H, KNS_L, KNS_LD>;
-template cudaError_t launch_sdf_cfg<InstCfg>(const GridView &, const float *, int64_t, float *, float *, float *,
-                                             cudaStream_t);
 template cudaError_t launch_occ_cfg<InstCfg>(const GridView &, float, uint32_t *, cudaStream_t);
 template cudaError_t launch_refine_cfg<InstCfg>(const GridView &, const WaveArgs &, int, cudaStream_t);
 #endif

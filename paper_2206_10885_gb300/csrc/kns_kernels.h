@@ -126,9 +126,23 @@ cudaError_t launch_trace_tc_cfg(const GridView &g, const WaveArgs &a, int sm_cou
 // pend_t[0] = the FP32 d at the ray's t), then their shading, one thread per ray.
 template <class C>
 cudaError_t launch_refine_cfg(const GridView &g, const WaveArgs &a, int sm_count, cudaStream_t s);
+// Scratch of a grouped field query of up to kPointsChunk points.
+constexpr int kPointsTile = 16;                // points per tile
+constexpr int64_t kPointsChunk = 1 << 22;      // points grouped at a time
+struct PointsScratch {
+    int *ctl;        // points placed, tiles made; the cells' counts follow
+    int *count;      // per cell: its points, then the start of its segment
+    int *rank;       // per point: its place in its cell
+    float4 *sorted;  // x, y, z, point number (bit pattern), by cell
+    int4 *tiles;     // cell, first sorted point, points
+};
+inline int64_t points_max_tiles(int64_t n, int64_t ncl) { return n / kPointsTile + (ncl < n ? ncl : n) + 1; }
 template <class C>
-cudaError_t launch_sdf_cfg(const GridView &g, const float *pts, int64_t n, float *sdf, float *feat, float *grad,
-                           cudaStream_t s);
+cudaError_t launch_points_direct_cfg(const GridView &g, const float *pts, int64_t n, float *sdf, float *feat,
+                                     float *grad, cudaStream_t s);
+template <class C>
+cudaError_t launch_points_tiles_cfg(const GridView &g, const PointsScratch &sc, int64_t n, float *sdf, float *feat,
+                                    float *grad, int sm_count, cudaStream_t s);
 template <class C>
 cudaError_t launch_occ_cfg(const GridView &g, float thresh, uint32_t *words, cudaStream_t s);
 
@@ -161,8 +175,13 @@ cudaError_t launch_wave_scatter(const WaveArgs &a, int cur, int blocks, cudaStre
 // Measured FP32 FMA (FLOP/s) and ex2 (operations/s) throughput of the device (kns_peak.cu).
 cudaError_t measure_peaks(int sm_count, cudaStream_t s, double *ffma_flops, double *mufu_ops);
 
-cudaError_t launch_sdf_f32(const Shape &sh, const GridView &g, const float *pts, int64_t n, float *sdf,
-                           float *feat, float *grad, cudaStream_t s);
+// Field query, one point per warp in the order given; or grouped by cell (launch_points_sort, then the tiles).
+cudaError_t launch_points_direct(const Shape &sh, const GridView &g, const float *pts, int64_t n, float *sdf,
+                                 float *feat, float *grad, cudaStream_t s);
+cudaError_t launch_points_sort(const GridView &g, const float *pts, int n, const PointsScratch &sc, int sm_count,
+                               cudaStream_t s);
+cudaError_t launch_points_tiles(const Shape &sh, const GridView &g, const PointsScratch &sc, int64_t n, float *sdf,
+                                float *feat, float *grad, int sm_count, cudaStream_t s);
 cudaError_t launch_occupancy_f32(const Shape &sh, const GridView &g, float thresh, uint32_t *words,
                                  cudaStream_t s);
 

@@ -8,6 +8,8 @@
 //          block-wide scan of its range (wave_scan_final_kernel) -- no block waits for another.
 // scatter: each sample goes to off[cell] + (its rank among the wave's samples of that cell);
 //          lanes of a warp that share a cell take consecutive slots with one atomic.
+#include <algorithm>
+
 #include "kns_wave.cuh"
 
 namespace kns {
@@ -246,6 +248,64 @@ cudaError_t launch_wave_scan(const WaveArgs &a, int cur, cudaStream_t s) {
 
 cudaError_t launch_wave_scatter(const WaveArgs &a, int cur, int blocks, cudaStream_t s) {
     wave_scatter_kernel<<<blocks, 256, 0, s>>>(a, cur);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------- field-query points by cell
+// Three passes: a count per cell (each point keeps its rank in its cell), a segment of `sorted` and tiles of
+// `tile` points for every non-empty cell, and the scatter.  The segments lie in any order, so the blocks of
+// the second pass only add their totals to two cursors.  Bound by the points' 12 bytes, read twice.
+__global__ void __launch_bounds__(256) points_count_kernel(GridView g, const float *__restrict__ pts, int n,
+                                                           PointsScratch s) {
+    const int lane = threadIdx.x & 31, bound = (n + 31) & ~31;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < bound; i += gridDim.x * blockDim.x) {
+        const unsigned m = __ballot_sync(FULL, i < n);
+        if (i < n) {
+            const int c = cell_of(g, pts[3 * (int64_t)i], pts[3 * (int64_t)i + 1], pts[3 * (int64_t)i + 2]);
+            const unsigned grp = __match_any_sync(m, c);
+            const int leader = __ffs(grp) - 1;
+            int base = 0;
+            if (lane == leader) base = atomicAdd(s.count + c, __popc(grp));
+            base = __shfl_sync(grp, base, leader);
+            s.rank[i] = base + __popc(grp & lanemask_lt());
+        }
+    }
+}
+
+__global__ void __launch_bounds__(SCAN_THREADS) points_segment_kernel(PointsScratch s, int ncl, int tile) {
+    __shared__ int wa[32], wb[32], base[2];
+    const int c = blockIdx.x * SCAN_THREADS + threadIdx.x;
+    const int n = c < ncl ? s.count[c] : 0, nt = (n + tile - 1) / tile;
+    int incl_n = n, incl_t = nt;
+    block_scan2(incl_n, incl_t, wa, wb);
+    if (threadIdx.x == SCAN_THREADS - 1) {
+        base[0] = incl_n ? atomicAdd(s.ctl, incl_n) : 0;
+        base[1] = incl_t ? atomicAdd(s.ctl + 1, incl_t) : 0;
+    }
+    __syncthreads();
+    if (n == 0) return;
+    const int first = base[0] + incl_n - n;
+    int t = base[1] + incl_t - nt;
+    s.count[c] = first;  // the scatter's segment starts
+    for (int i = 0; i < n; i += tile) s.tiles[t++] = make_int4(c, first + i, min(tile, n - i), 0);
+}
+
+__global__ void __launch_bounds__(256) points_scatter_kernel(GridView g, const float *__restrict__ pts, int n,
+                                                             PointsScratch s) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const float x = pts[3 * (int64_t)i], y = pts[3 * (int64_t)i + 1], z = pts[3 * (int64_t)i + 2];
+        s.sorted[s.count[cell_of(g, x, y, z)] + s.rank[i]] = make_float4(x, y, z, __int_as_float(i));
+    }
+}
+
+cudaError_t launch_points_sort(const GridView &g, const float *pts, int n, const PointsScratch &sc, int sm_count,
+                               cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(sc.ctl, 0, sizeof(int) * (2 + (size_t)g.ncl), s);  // ctl, then count
+    if (e != cudaSuccess) return e;
+    const int blocks = std::min(sm_count * 8, (n + 255) / 256);
+    points_count_kernel<<<blocks, 256, 0, s>>>(g, pts, n, sc);
+    points_segment_kernel<<<(g.ncl + SCAN_THREADS - 1) / SCAN_THREADS, SCAN_THREADS, 0, s>>>(sc, g.ncl, kPointsTile);
+    points_scatter_kernel<<<blocks, 256, 0, s>>>(g, pts, n, sc);
     return cudaGetLastError();
 }
 
