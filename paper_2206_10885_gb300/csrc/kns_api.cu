@@ -91,6 +91,7 @@ struct kns_ctx {
     size_t ev_used = 0;
     int cur_round = -1;                    // round being enqueued (tags timing marks)
     std::vector<int> round_live;           // samples queued per round of the last render (-1: not read)
+    int round0 = 0;                        // its last batch's first round
     // stream-ordered scratch of grouped field queries: calls on several streams each get their own
     cudaMemPool_t pool = nullptr;
 };
@@ -1145,11 +1146,16 @@ kns_status render_views_impl(kns_ctx *ctx, const kns_grid *grid, const std::vect
     // puts it on its round's pending list: the advance kernel of round k walks those rays to their
     // next occupied voxel on the side stream while round k + 1 runs (after round k + 1's scan has
     // cleared the counters it adds to) and they rejoin in round k + 2, whose scan waits for it.  So a
-    // ray's budget of max_steps steps takes at most 2 max_steps rounds.  The host reads, for round
-    // k - 2, its live count and round k - 3's pending count before launching round k, and stops when
-    // both are zero (rounds k - 1 and k then hold nothing), so it runs at most two rounds ahead.
+    // ray's budget of max_steps steps takes at most 2 max_steps rounds.  Round k's live count and round
+    // k - 1's pending count are known after its scan, so the host has launched round k before it reads
+    // them and launches round k + 1 while round k's tiles run; it stops when both are zero, or when the
+    // round is small enough for the tail (which leaves nothing to a later round) and nothing is pending.
+    // A render of no more rays than that takes one round and no host read.  (An empty round costs about
+    // 30 us of launches; reading two rounds late, every render ran two of them: four 64 x 64 views took
+    // 240 us and take 163, a 200 x 150 path trace of 8 paths and 4 traces 1.47 ms and 1.26.)
     int last_adv = -1;  // the last round whose advance kernel was launched
-    const int round0 = (int)ctx->round_live.size();  // rounds of earlier batches of this call
+    bool small = !cfg.bf16 && rays <= cfg.tail_rays;  // the round at hand is known to be the tail's, and the last
+    const int round0 = ctx->round0 = (int)ctx->round_live.size();  // rounds of earlier batches of this call
     if (e == cudaSuccess && cfg.bf16 && cfg.persistent) {  // every round on the device, one launch
         a.btile = 128;
         const int tm = timing_begin(ctx, cfg.timing, kTEvalBF16, s);
@@ -1164,10 +1170,6 @@ kns_status render_views_impl(kns_ctx *ctx, const kns_grid *grid, const std::vect
     for (int k = 0; k < 2 * max_steps + 2 && e == cudaSuccess && !(cfg.bf16 && cfg.persistent); ++k) {
         const int cur = k & 1;
         if (k >= 2) {
-            e = cudaEventSynchronize(ctx->ev_live[(k - 2) & 3]);
-            const int *hl = ctx->h_live + 2 * ((k - 2) & 3);
-            if (e == cudaSuccess) ctx->round_live[round0 + k - 2] = hl[0];
-            if (e != cudaSuccess || (hl[0] == 0 && hl[1] == 0)) break;
             // round k - 2's advance added to this round's counters
             e = cudaStreamWaitEvent(s, ctx->ev_adv[k & 1], 0);
             if (e != cudaSuccess) break;
@@ -1204,11 +1206,19 @@ kns_status render_views_impl(kns_ctx *ctx, const kns_grid *grid, const std::vect
             tm = timing_begin(ctx, cfg.timing, kTEvalF32, s);
             if (e == cudaSuccess) e = kns::launch_wave_tail(grid->shape, grid->view, a, cur, ctx->sm_count, s);
             timing_end(ctx, tm, s);
-        } else if (e == cudaSuccess) {  // FP32 tiles and the one-warp-per-ray tail
+        } else if (e == cudaSuccess) {  // FP32 tiles and the tail; the tail alone where it will take the round
             tm = timing_begin(ctx, cfg.timing, kTEvalF32, s);
-            e = kns::launch_wave_eval(grid->shape, grid->view, a, cur, eval_blocks, cfg.block_mode, ctx->sm_count, s);
+            e = small ? kns::launch_wave_tail(grid->shape, grid->view, a, cur, ctx->sm_count, s)
+                      : kns::launch_wave_eval(grid->shape, grid->view, a, cur, eval_blocks, cfg.block_mode,
+                                              ctx->sm_count, s);
             timing_end(ctx, tm, s);
         }
+        if (e != cudaSuccess || small) break;
+        e = cudaEventSynchronize(ctx->ev_live[k & 3]);
+        if (e != cudaSuccess) break;
+        ctx->round_live[round0 + k] = hl[0];
+        if (hl[1] == 0 && (hl[0] == 0 || hl[0] <= a.tail_max)) break;
+        small = hl[0] + hl[1] <= a.tail_max;  // the next round holds these pending rays alone: its tail ends it
     }
     ctx->cur_round = -1;
     // the side stream's last advance joins before the shading (it found nothing: the rounds ended)
@@ -1233,6 +1243,8 @@ kns_status render_views_impl(kns_ctx *ctx, const kns_grid *grid, const std::vect
         ctx->stats.samples_bf16 += (int64_t)hc.samples_bf16;
         ctx->stats.samples_tail += (int64_t)hc.samples_tail;
         ctx->stats.refined += hc.n_refine;
+        for (int k = round0; k < (int)ctx->round_live.size(); ++k)  // counts copied but not waited for
+            if (ctx->round_live[k] < 0) ctx->round_live[k] = ctx->h_live[2 * ((k - round0) & 3)];
     }
     return KNS_OK;
 }
@@ -1523,7 +1535,7 @@ kns_status kns_get_round_trace(kns_ctx *ctx, kns_round_info *out, int32_t max_ro
     const int n = (int)ctx->round_live.size();
     // the last rounds' counts were copied to the pinned ring but not read by the render loop
     for (int k = std::max(0, n - 4); k < n; ++k)
-        if (ctx->round_live[k] < 0) ctx->round_live[k] = ctx->h_live[2 * (k & 3)];
+        if (ctx->round_live[k] < 0) ctx->round_live[k] = ctx->h_live[2 * ((k - ctx->round0) & 3)];
     *n_rounds = n;
     for (int k = 0; k < std::min(n, (int)max_rounds); ++k) out[k] = kns_round_info{ctx->round_live[k], 0.f, 0.f, 0.f, 0.f, 0};
     for (const auto &m : ctx->ev_marks) {
@@ -1703,10 +1715,6 @@ extern "C" kns_status kns_render_noalloc(kns_ctx *ctx, const kns_grid *grid, con
     const int eval_blocks = ctx->sm_count * kRenderBlocksPerSM, scatter_blocks = ctx->sm_count * 4;
     for (int k = 0; k < max_steps && e == cudaSuccess; ++k) {
         const int cur = k & 1;
-        if (k >= 2) {
-            e = cudaEventSynchronize(ctx->ev_live[(k - 2) & 3]);
-            if (e != cudaSuccess || ctx->h_live[2 * ((k - 2) & 3)] == 0) break;
-        }
         e = kns::launch_wave_scan(a, cur, s);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(ctx->h_live + 2 * (k & 3), &a.ctrl->n_live[cur], sizeof(int), cudaMemcpyDeviceToHost,
@@ -1714,6 +1722,10 @@ extern "C" kns_status kns_render_noalloc(kns_ctx *ctx, const kns_grid *grid, con
         if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_live[k & 3], s);
         if (e == cudaSuccess) e = kns::launch_wave_scatter(a, cur, scatter_blocks, s);
         if (e == cudaSuccess) e = kns::launch_wave_eval(grid->shape, grid->view, a, cur, eval_blocks, 0, ctx->sm_count, s);
+        // the tail takes a round of at most tail_max rays, and with it the last ones
+        if (e != cudaSuccess || rays <= a.tail_max) break;
+        e = cudaEventSynchronize(ctx->ev_live[k & 3]);
+        if (e != cudaSuccess || ctx->h_live[2 * (k & 3)] <= a.tail_max) break;
     }
     if (e == cudaSuccess) {
         // the same shading as kns_render (hits sorted by cell, block tiles)
