@@ -1,16 +1,19 @@
 // kns_train_tile.cu -- the grouped MLP kernels of the training step: SDF and colour MLPs of one cell
-// evaluated, and differentiated, on tiles of 128 same-cell records as register-blocked block GEMMs.
+// evaluated, and differentiated, on warp tiles of same-cell records.
 //
-// A block of 256 threads takes a chunk (up to 4096 records of one cell, from the counting sort),
-// stages the cell's weights in shared memory (forward layers k-major, backward layers row-major) and
-// walks the chunk in tiles of 128 records.  Activations and deltas of a tile live in shared memory
-// as rows of 128 records (row stride 132 floats).  Every dense layer, forward (A_l = act(W A_{l-1} +
-// b)) and backward (D_l = (W^T D_{l+1}) . act'(A_l)), is a [32 x K] by [K x 128] product in which a
-// thread owns 4 outputs x 4 records: per k one warp-uniform float4 of weights and one float4 of
-// activations feed 16 FMAs.  The weight gradient of the tile, dW_l = D_l A_{l-1}^T summed over the
-// tile's records, is formed by thread-owned 4 x 4 blocks of (output, input) entries that accumulate
-// in registers over every tile of the chunk and are added to the global gradient once per chunk;
-// bias gradients come out of the same sums through a constant-one input row.
+// A block takes a chunk (up to 4096 records of one cell, from the counting sort), stages the cell's weights in
+// shared memory (forward layers k-major, backward layers row-major), and its warps walk the chunk in tiles of
+// 32 records (16 for the sample centres), each on rows of its own: every dense layer, forward (A_l = act(W
+// A_{l-1} + b)) and backward (D_l = (W^T D_{l+1}) . act'(A_l)), is a product of the warp's 8 x 4 lanes
+// (kns_warp.cuh), so no barrier stands between layers, only around a chunk.  The weight gradient of a tile, dW_l =
+// D_l A_{l-1}^T summed over its records, accumulates in the lanes' registers over the whole chunk, and the
+// block adds its warps' sums to the global gradient once per chunk.
+//
+// What bounds them is the FP32 pipe and the loads that feed it.  Block tiles of 128 records (a barrier per layer;
+// for each layer's weight gradient only the 72 threads that held its entries at work) took, per step of 65,536 rays
+// x 96 samples and 16,384 eikonal points on a GB300: difference points forward 7.1 ms, centres forward 2.5,
+// centres backward 10.6, difference points backward 28.6 ms; now 6.3, 2.2, 7.2 and 24.7 ms (the step 51.3 -> 42.4
+// ms; 1,024 rays 3.0 -> 2.5 ms).
 //
 // Kernels: d at records (coarse samples and difference points); sample centres forward (d, z,
 // colour); sample centres backward (colour and SDF, writes the difference points' upstream);
@@ -21,6 +24,7 @@
 #include "kns_device.cuh"
 #include "kns_kernels.h"
 #include "kns_train.cuh"
+#include "kns_warp.cuh"
 
 namespace kns {
 namespace {
@@ -31,100 +35,15 @@ using train::fd_normal;
 using train::grid_for;
 using train::load3;
 
-constexpr int TPB = 256;     // threads per block
-constexpr int TILE = 128;    // records per tile
-constexpr int RS = TILE + 4;  // shared row stride (floats)
 constexpr int PE_L = 4;
 
-// ------------------------------------------------------------------ shared weight layout
-// [forward SDF | forward colour | backward SDF | backward colour], every block 16-byte aligned:
-//   forward SDF:  T0[28][32] (T0[k][o] = W0[o][k], row 27 zero), b0[32]; per hidden layer l = 1..H-1
-//                 Tl[32][32], bl[32]; To[32][16] (To[k][o] = Wo[o][k]), bo[16]
-//   forward colour: C0t[36][32] (k < 33), c0[32], C1t[32][4] (c < 3), c1[4]
-//   backward SDF: W_l[32][32] row-major (l = 1..H-1), Wo[16][32]
-//   backward colour: Wc0[32][36] row-major (i < 33), Wc1[4][32] (row 3 zero)
+// ------------------------------------------------------------------ canonical offsets in a cell
 template <int H>
 struct WL {
-    static constexpr int T0 = 0, b0 = 28 * 32, HL = 32 * 32 + 32;
-    __host__ __device__ static constexpr int Tl(int l) { return b0 + 32 + (l - 1) * HL; }
-    __host__ __device__ static constexpr int bl(int l) { return Tl(l) + 1024; }
-    static constexpr int To = b0 + 32 + (H - 1) * HL, bo = To + 512, FS = bo + 16;
-    static constexpr int C0t = FS, c0 = C0t + 36 * 32, C1t = c0 + 32, c1 = C1t + 128, FC = c1 + 4;
-    __host__ __device__ static constexpr int Wr(int l) { return FC + (l - 1) * 1024; }
-    static constexpr int Wo = FC + (H - 1) * 1024, BS = Wo + 512;
-    static constexpr int Wc0 = BS, Wc1 = Wc0 + 32 * 36, END = Wc1 + 128;
-    // canonical offsets (per cell)
+    static constexpr int HL = 32 * 32 + 32;
     static constexpr int cW0 = 0, cb0 = 27 * 32, cH = cb0 + 32;
     static constexpr int cWo = cH + (H - 1) * HL, cbo = cWo + 512, cC0 = cbo + 16;
     static constexpr int cc0 = cC0 + 33 * 32, cC1 = cc0 + 32, cc1 = cC1 + 96;
-};
-
-// canonical index of shared weight slot j (-1: zero)
-template <int H>
-__device__ int canon_slot(int j) {
-    using L = WL<H>;
-    if (j < L::b0) {  // T0[k][o]
-        const int k = j >> 5, o = j & 31;
-        return k < 27 ? L::cW0 + o * 27 + k : -1;
-    }
-    if (j < L::To) {
-        if (j < L::Tl(1)) return L::cb0 + (j - L::b0);
-        const int r = j - L::Tl(1), l = r / L::HL, u = r - l * L::HL;
-        if (u < 1024) return L::cH + l * L::HL + (u & 31) * 32 + (u >> 5);  // Tl[k][o] = W[o][k]
-        return L::cH + l * L::HL + u;                                        // bias
-    }
-    if (j < L::bo) {
-        const int u = j - L::To, k = u >> 4, o = u & 15;
-        return L::cWo + o * 32 + k;
-    }
-    if (j < L::FS) return L::cbo + (j - L::bo);
-    if (j < L::c0) {
-        const int u = j - L::C0t, k = u >> 5, o = u & 31;
-        return k < 33 ? L::cC0 + o * 33 + k : -1;
-    }
-    if (j < L::C1t) return L::cc0 + (j - L::c0);
-    if (j < L::c1) {
-        const int u = j - L::C1t, k = u >> 2, c = u & 3;
-        return c < 3 ? L::cC1 + c * 32 + k : -1;
-    }
-    if (j < L::FC) return j - L::c1 < 3 ? L::cc1 + (j - L::c1) : -1;
-    if (j < L::Wo) {
-        const int r = j - L::FC, l = r >> 10, u = r & 1023;
-        return L::cH + l * L::HL + u;  // row-major as stored
-    }
-    if (j < L::BS) return L::cWo + (j - L::Wo);
-    if (j < L::Wc1) {
-        const int u = j - L::Wc0, o = u / 36, i = u - o * 36;
-        return i < 33 ? L::cC0 + o * 33 + i : -1;
-    }
-    const int u = j - L::Wc1, c = u >> 5, k = u & 31;
-    return c < 3 ? L::cC1 + c * 32 + k : -1;
-}
-
-template <int H>
-__device__ __forceinline__ void load_slots(const float *__restrict__ cw, float *sw, int j0, int j1) {
-    for (int j = j0 + (int)threadIdx.x; j < j1; j += TPB) {
-        const int c = canon_slot<H>(j);
-        sw[j] = c >= 0 ? __ldg(cw + c) : 0.f;
-    }
-}
-
-// ------------------------------------------------------------------ tile rows
-// A0 (28: encoding + one), A_l (36: 32 + one + 3 zero), D_l (32), Dout (16: d and z deltas),
-// then the colour rows: the d output row, U (36: z, n, gamma(v), one, 2 zero), Hc (36), Dh (32), Dc (4)
-template <int H>
-struct RL {
-    static constexpr int A0 = 0;
-    __host__ __device__ static constexpr int A(int l) { return 28 + (l - 1) * 36; }
-    __host__ __device__ static constexpr int D(int l) { return 28 + 36 * H + (l - 1) * 32; }
-    static constexpr int Dout = 28 + 68 * H;
-    // difference records backward in place: D_l over A_l (rows 0..31; the one row stays), then Dout
-    static constexpr int DoutF = 28 + 36 * H, FDI_ROWS = DoutF + 4;
-    static constexpr int Ud = Dout + 16, U = Ud + 1, Hc = U + 36, Dh = Hc + 36, Dc = Dh + 32;
-    static constexpr int C_ROWS = Dc + 4;
-    // forward-only kernels: A0, two ping-pong layers, then (centres) the output row, U and Hc
-    static constexpr int P = 28, Q = P + 32, F_ROWS = Q + 32;
-    static constexpr int FUd = Q + 32, FU = FUd + 1, FHc = FU + 36, FC_ROWS = FHc + 32;
 };
 
 // ------------------------------------------------------------------ activations
@@ -138,648 +57,663 @@ __device__ __forceinline__ float dsoftplus_act(float a, float beta) {
 }
 __device__ __forceinline__ float sigm(float s) { return 1.f / (1.f + __expf(-s)); }
 
-// ------------------------------------------------------------------ block GEMMs
-// thread blocking: outputs o0 .. o0+3 (o0 = 4 warp), records r0 .. r0+3 (r0 = 4 lane)
-__device__ __forceinline__ int o0_32() { return (threadIdx.x >> 5) * 4; }
-__device__ __forceinline__ int r0_t() { return (threadIdx.x & 31) * 4; }
+// ------------------------------------------------------------------ records on warps
+// The kernels of the difference points and coarse samples (151 M records in a step of 2^18 rays) work on warp
+// tiles: a warp takes 32 records of the chunk's cell through every layer on its own rows in shared memory
+// (kns_warp.cuh's map: 8 records x 4 units a lane), with no barrier but those around the cell's weights,
+// which the block's warps share.
+constexpr int WT = 32;                 // records per warp tile
+constexpr int WRS = row_stride(WT);    // row stride (floats)
+constexpr int WTS = 36;                // row stride of transposed weights: the transposing stores conflict less
 
-// acc[i][j] += sum_k Wk[k WS + o0 + i] X[k RS + r0 + j]
-template <int K, int WS>
-__device__ __forceinline__ void mm32(const float *Wk, const float *X, float (&acc)[4][4]) {
-    const float *w = Wk + o0_32();
-    const float *x = X + r0_t();
-#pragma unroll 4
-    for (int k = 0; k < K; ++k) {
-        const float4 wv = *reinterpret_cast<const float4 *>(w + k * WS);
-        const float4 xv = *reinterpret_cast<const float4 *>(x + k * RS);
-        const float wa[4] = {wv.x, wv.y, wv.z, wv.w}, xa[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(wa[i], xa[j], acc[i][j]);
+// weights of one cell in shared memory (floats): per layer T_l[k][o] (stride WTS) and b_l; the row-major
+// hidden layers the deltas run back through; the d row and its bias
+template <int H>
+struct WW {
+    static constexpr int K0 = 28;
+    __host__ __device__ static constexpr int T(int l) { return l == 0 ? 0 : K0 * WTS + 32 + (l - 1) * (32 * WTS + 32); }
+    __host__ __device__ static constexpr int b(int l) { return T(l) + (l == 0 ? K0 : 32) * WTS; }
+    static constexpr int wo = T(H), bo = wo + 32, FEND = bo + 4;
+    __host__ __device__ static constexpr int R(int l) { return FEND + (l - 1) * 1024; }
+    static constexpr int END = FEND + (H - 1) * 1024;
+};
+
+// the cell's canonical SDF weights into sw (every thread of the block; nt threads)
+template <int H, bool BACKWARD>
+__device__ __forceinline__ void load_cell(const float *__restrict__ cw, float *sw, int nt) {
+    using L = WL<H>;
+    using S = WW<H>;
+    const int tid = threadIdx.x;
+    for (int j = tid; j < 27 * 32; j += nt) sw[S::T(0) + (j % 27) * WTS + j / 27] = __ldg(cw + L::cW0 + j);
+    if (tid < 32) {
+        sw[S::T(0) + 27 * WTS + tid] = 0.f;
+        sw[S::b(0) + tid] = __ldg(cw + L::cb0 + tid);
+        sw[S::wo + tid] = __ldg(cw + L::cWo + tid);
+        if (tid == 0) sw[S::bo] = __ldg(cw + L::cbo);
     }
-}
-
-// 16 outputs: o0 = 2 warp, outputs o0, o0+1; acc[i][j] += sum_k Wk[k 16 + o0 + i] X[k RS + r0 + j]
-template <int K>
-__device__ __forceinline__ void mm16(const float *Wk, const float *X, float (&acc)[2][4]) {
-    const float *w = Wk + (threadIdx.x >> 5) * 2;
-    const float *x = X + r0_t();
-#pragma unroll 4
-    for (int k = 0; k < K; ++k) {
-        const float2 wv = *reinterpret_cast<const float2 *>(w + k * 16);
-        const float4 xv = *reinterpret_cast<const float4 *>(x + k * RS);
-        const float xa[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            acc[0][j] = fmaf(wv.x, xa[j], acc[0][j]);
-            acc[1][j] = fmaf(wv.y, xa[j], acc[1][j]);
+    for (int l = 1; l < H; ++l) {
+        const float *src = cw + L::cH + (l - 1) * L::HL;
+        for (int j = tid; j < 1024; j += nt) {
+            const float v = __ldg(src + j);
+            sw[S::T(l) + (j & 31) * WTS + (j >> 5)] = v;
+            if (BACKWARD) sw[S::R(l) + j] = v;
         }
+        if (tid < 32) sw[S::b(l) + tid] = __ldg(src + 1024 + tid);
     }
 }
 
-__device__ __forceinline__ void init_bias(const float *b, float (&acc)[4][4]) {
-    const float4 bv = *reinterpret_cast<const float4 *>(b + o0_32());
-    const float ba[4] = {bv.x, bv.y, bv.z, bv.w};
+// encoding of record `lane` (Eq. 1) into column lane of rows E; row 27 is zero
+__device__ __forceinline__ void encode_record(float *E, int lane, float x, float y, float z) {
+    float in[28];
+    encode3<PE_L>(x, y, z, in);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = ba[i];
-}
-__device__ __forceinline__ void zero(float (&acc)[4][4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-}
-__device__ __forceinline__ void store_rows(float *rows, int row0, const float (&v)[4][4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        *reinterpret_cast<float4 *>(rows + (row0 + o0_32() + i) * RS + r0_t()) =
-            make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
-}
-__device__ __forceinline__ void load_rows(const float *rows, int row0, float (&v)[4][4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float4 x = *reinterpret_cast<const float4 *>(rows + (row0 + o0_32() + i) * RS + r0_t());
-        v[i][0] = x.x;
-        v[i][1] = x.y;
-        v[i][2] = x.z;
-        v[i][3] = x.w;
-    }
-}
-
-// one SDF hidden layer: rows[dst] = softplus(W rows[src] + b)
-template <int K>
-__device__ __forceinline__ void hidden_layer(const float *Wk, const float *b, float *rows, int src, int dst,
-                                             float beta, float inv_beta) {
-    float acc[4][4];
-    init_bias(b, acc);
-    mm32<K, 32>(Wk, rows + src * RS, acc);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = softplus(acc[i][j], beta, inv_beta);
-    store_rows(rows, dst, acc);
-}
-
-// encoding of record column col into rows A0 .. A0+26, split between two threads: half 0 writes x
-// and frequencies 0, 1; half 1 frequencies 2, 3 (rows 3 + 6k + c: sin, 3 + 6k + 3 + c: cos)
-__device__ __forceinline__ void encode_half(float *rows, int a0, int col, int half, float x, float y, float z) {
-    const float p[3] = {x, y, z};
-    if (half == 0) {
-        rows[(a0 + 0) * RS + col] = x;
-        rows[(a0 + 1) * RS + col] = y;
-        rows[(a0 + 2) * RS + col] = z;
-    }
-#pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-        const int k = 2 * half + kk;
-        const float f = (float)(1 << k);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            float sn, cs;
-            sincospif(f * p[c], &sn, &cs);
-            rows[(a0 + 3 + 6 * k + c) * RS + col] = sn;
-            rows[(a0 + 6 + 6 * k + c) * RS + col] = cs;
-        }
-    }
+    for (int k = 0; k < 28; ++k) E[k * WRS + lane] = in[k];
 }
 
 // ------------------------------------------------------------------ forward: d at records
+constexpr int FW = 8;  // warps per block
 template <int H>
-__global__ void __launch_bounds__(TPB, 3) k_tile_eval_d(TrainArgs a, int k0, int k1, float *out) {
-    using L = WL<H>;
-    using R = RL<H>;
+__global__ void __launch_bounds__(32 * FW, 2) k_warp_eval_d(TrainArgs a, int k0, int k1, float *out) {
+    using S = WW<H>;
     extern __shared__ float4 smem4[];
-    float *rows = reinterpret_cast<float *>(smem4);
-    float *sw = rows + R::F_ROWS * RS;
-    __shared__ int s_rec[TILE];
-    const int tid = threadIdx.x;
+    float *sw = reinterpret_cast<float *>(smem4);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float *rows = sw + S::FEND + warp * 32 * WRS;  // a layer overwrites its input
     const int c0 = a.chunk_off[k0], total = a.chunk_off[k1] - c0;
-    constexpr int last = (H % 2 == 1) ? R::P : R::Q;  // A0 -> P -> Q -> P ...
+    auto act = [&](float v, int, int) { return softplus(v, a.beta, a.inv_beta); };
     for (int ci = blockIdx.x; ci < total; ci += gridDim.x) {
         const int key = chunk_key(a.chunk_off, k0, k1, c0 + ci);
         const int j = c0 + ci - a.chunk_off[key];
         const int beg = a.off[key] + j * CHUNK, end = min(beg + CHUNK, a.off[key + 1]);
         __syncthreads();
-        load_slots<H>(a.params + (int64_t)key * a.p_cell, sw, 0, L::FS);
-        for (int tb = beg; tb < end; tb += TILE) {
-            {
-                const int col = tid & (TILE - 1), i = tb + col;
-                float4 r = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
-                if (i < end) r = a.sorted[i];
-                if (tid < TILE) s_rec[tid] = __float_as_int(r.w);
-                encode_half(rows, R::A0, col, tid >> 7, r.x, r.y, r.z);
-            }
-            __syncthreads();
-            hidden_layer<27>(sw + L::T0, sw + L::b0, rows, R::A0, R::P, a.beta, a.inv_beta);
+        load_cell<H, false>(a.params + (int64_t)key * a.p_cell, sw, 32 * FW);
+        __syncthreads();
+        for (int tb = beg + WT * warp; tb < end; tb += WT * FW) {
+            float4 r = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+            if (tb + lane < end) r = a.sorted[tb + lane];
+            encode_record(rows, lane, r.x, r.y, r.z);
+            __syncwarp();
+            TileMap<32, WT> m(lane);
+            m.bias_shared(sw + S::b(0));
+            m.template mm_shared<28>(sw + S::T(0), WTS, rows, WRS);
+            __syncwarp();  // every lane has read the input before it is overwritten
+            m.store(rows, WRS, act);
+            __syncwarp();
 #pragma unroll
             for (int l = 1; l < H; ++l) {
-                __syncthreads();
-                hidden_layer<32>(sw + L::Tl(l), sw + L::bl(l), rows, (l % 2) ? R::P : R::Q, (l % 2) ? R::Q : R::P,
-                                 a.beta, a.inv_beta);
+                m.bias_shared(sw + S::b(l));
+                m.template mm_shared<32>(sw + S::T(l), WTS, rows, WRS);
+                __syncwarp();
+                m.store(rows, WRS, act);
+                __syncwarp();
             }
-            __syncthreads();
-            if (tid < TILE && s_rec[tid] >= 0) {
-                float d = sw[L::bo];
+            float d = sw[S::bo];
 #pragma unroll 8
-                for (int k = 0; k < 32; ++k) d = fmaf(sw[L::To + k * 16], rows[(last + k) * RS + tid], d);
-                out[s_rec[tid]] = d;
+            for (int k = 0; k < 32; ++k) d = fmaf(sw[S::wo + k], rows[k * WRS + lane], d);
+            const int rec = __float_as_int(r.w);
+            if (rec >= 0) out[rec] = d;
+            __syncwarp();
+        }
+    }
+}
+
+// ------------------------------------------------------------------ backward of the difference points
+// Per warp tile: the forward layers recomputed (rows E, A_1 .. A_H), then from the output back, each layer's
+// weight gradient while its inputs are still in their rows and the deltas D_l over A_l.  The weight gradients
+// of the whole chunk stay in registers -- lane (og, ig) = (lane / 8, lane % 8) owns outputs og + 4 i and inputs
+// ig + 8 j of every layer, 12 loads of 16 bytes for 128 FMAs -- and are summed over the block's warps in shared
+// memory and added to the global gradient once per chunk.
+constexpr int BW = 5;  // warps per block, two blocks per SM
+template <int H>
+struct WRows {
+    __host__ __device__ static constexpr int A(int l) { return 32 * l; }  // A(0): the encoding
+    static constexpr int G = 32 * (H + 1), ROWS = G + 1;                  // G: the upstream of d
+};
+
+// acc[i][j] += sum over the tile's records of D[og + 4 i] A[ig + 8 j]
+__device__ __forceinline__ void grad_tile32(const float *D, const float *A, float (&acc)[8][4], int lane) {
+    const float *d = D + (lane >> 3) * WRS, *x = A + (lane & 7) * WRS;
+#pragma unroll 2
+    for (int r = 0; r < WT; r += 4) {
+        float4 xv[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) xv[j] = *reinterpret_cast<const float4 *>(x + 8 * j * WRS + r);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 dv = *reinterpret_cast<const float4 *>(d + 4 * i * WRS + r);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float s = acc[i][j];
+                s = fmaf(dv.x, xv[j].x, s);
+                s = fmaf(dv.y, xv[j].y, s);
+                s = fmaf(dv.z, xv[j].z, s);
+                s = fmaf(dv.w, xv[j].w, s);
+                acc[i][j] = s;
             }
+        }
+    }
+}
+// sum over the tile's records of row `lane` of X times g (NULL: 1)
+__device__ __forceinline__ float row_sum32(const float *X, const float *g, int lane) {
+    float s = 0.f;
+#pragma unroll
+    for (int r = 0; r < WT; r += 4) {
+        const float4 x = *reinterpret_cast<const float4 *>(X + lane * WRS + r);
+        if (g) {
+            const float4 y = *reinterpret_cast<const float4 *>(g + r);
+            s = fmaf(x.x, y.x, s);
+            s = fmaf(x.y, y.y, s);
+            s = fmaf(x.z, y.z, s);
+            s = fmaf(x.w, y.w, s);
+        } else {
+            s += (x.x + x.y) + (x.z + x.w);
+        }
+    }
+    return s;
+}
+
+template <int H>
+__global__ void __launch_bounds__(32 * BW, 2) k_warp_fd_backward(TrainArgs a) {
+    using L = WL<H>;
+    using S = WW<H>;
+    using R = WRows<H>;
+    constexpr int NT = 32 * BW;
+    static_assert(R::ROWS * WRS >= L::cbo + 1, "a warp's rows must hold its gradient");
+    extern __shared__ float4 smem4[];
+    float *sw = reinterpret_cast<float *>(smem4);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float *all = sw + S::END, *rows = all + warp * R::ROWS * WRS, *gr = rows + R::G * WRS;
+    const int c0 = a.chunk_off[0], total = a.chunk_off[a.NC] - c0;
+    auto act = [&](float v, int, int) { return softplus(v, a.beta, a.inv_beta); };
+    for (int ci = blockIdx.x; ci < total; ci += gridDim.x) {
+        const int cell = chunk_key(a.chunk_off, 0, a.NC, c0 + ci);
+        const int j = c0 + ci - a.chunk_off[cell];
+        const int beg = a.off[cell] + j * CHUNK, end = min(beg + CHUNK, a.off[cell + 1]);
+        __syncthreads();
+        load_cell<H, true>(a.params + (int64_t)cell * a.p_cell, sw, NT);
+#pragma unroll
+        for (int k = 27; k < 32; ++k) rows[k * WRS + lane] = 0.f;  // inputs past the encoding
+        __syncthreads();
+        float dw[H][8][4], db[H], dwo = 0.f, dbo = 0.f;
+#pragma unroll
+        for (int l = 0; l < H; ++l) {
+            db[l] = 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) dw[l][i][k] = 0.f;
+        }
+        for (int tb = beg + WT * warp; tb < end; tb += WT * BW) {
+            {
+                float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+                float g = 0.f;
+                if (tb + lane < end) {
+                    r = a.sorted[tb + lane];
+                    g = a.g_fd[__float_as_int(r.w)];
+                }
+                encode_record(rows, lane, r.x, r.y, r.z);
+                gr[lane] = g;
+                dbo += g;
+            }
+            __syncwarp();
+            TileMap<32, WT> m(lane);
+            m.bias_shared(sw + S::b(0));
+            m.template mm_shared<28>(sw + S::T(0), WTS, rows, WRS);
+            m.store(rows + R::A(1) * WRS, WRS, act);
+            __syncwarp();
+#pragma unroll
+            for (int l = 1; l < H; ++l) {
+                m.bias_shared(sw + S::b(l));
+                m.template mm_shared<32>(sw + S::T(l), WTS, rows + R::A(l) * WRS, WRS);
+                m.store(rows + R::A(l + 1) * WRS, WRS, act);
+                __syncwarp();
+            }
+            dwo += row_sum32(rows + R::A(H) * WRS, gr, lane);
+            __syncwarp();
+            {  // D_H = w_o g . softplus'(A_H)
+                float *own = rows + R::A(H) * WRS;
+                m.zero();
+                m.store(own, WRS, [&](float, int u, int s) {
+                    return sw[S::wo + u] * gr[s] * dsoftplus_act(own[u * WRS + s], a.beta);
+                });
+            }
+            __syncwarp();
+#pragma unroll
+            for (int l = H - 1; l >= 1; --l) {  // hidden layer l's weight gradient, then D_l over A_l
+                const float *D = rows + R::A(l + 1) * WRS;
+                float *own = rows + R::A(l) * WRS;
+                grad_tile32(D, own, dw[l], lane);
+                db[l] += row_sum32(D, nullptr, lane);
+                m.zero();
+                m.template mm_shared<32>(sw + S::R(l), 32, D, WRS);
+                __syncwarp();  // A_l has been read
+                m.store(own, WRS, [&](float v, int u, int s) { return v * dsoftplus_act(own[u * WRS + s], a.beta); });
+                __syncwarp();
+            }
+            grad_tile32(rows + R::A(1) * WRS, rows, dw[0], lane);
+            db[0] += row_sum32(rows + R::A(1) * WRS, nullptr, lane);
+            __syncwarp();
+        }
+        // the chunk's gradient: each warp's in its rows, canonical order; then summed over the warps
+        __syncwarp();
+        const int og = lane >> 3, ig = lane & 7;
+#pragma unroll
+        for (int l = 0; l < H; ++l) {
+            const int K = l == 0 ? 27 : 32, cW = l == 0 ? L::cW0 : L::cH + (l - 1) * L::HL;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (ig + 8 * k < K) rows[cW + (og + 4 * i) * K + ig + 8 * k] = dw[l][i][k];
+            rows[cW + 32 * K + lane] = db[l];
+        }
+        rows[L::cWo + lane] = dwo;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dbo += __shfl_xor_sync(0xffffffffu, dbo, o);
+        if (lane == 0) rows[L::cbo] = dbo;
+        __syncthreads();
+        const int nw = min(BW, (end - beg + WT - 1) / WT);  // warps that had a tile
+        float *gcell = a.grad + (int64_t)cell * a.p_cell;
+        for (int e = tid; e < L::cWo + 33; e += NT) {
+            const int q = e < L::cWo + 32 ? e : L::cbo;
+            float v = 0.f;
+            for (int w = 0; w < nw; ++w) v += all[w * R::ROWS * WRS + q];
+            if (v != 0.f) atomicAdd(gcell + q, v);
         }
     }
 }
 
 // ------------------------------------------------------------------ sample centres
-// colour input rows U: z (0..14), n (15..17), gamma_2(v) (18..32), one (33), zero (34, 35)
-__device__ __forceinline__ void centre_inputs(const TrainArgs &a, float *rows, int u, int col, int64_t q) {
-    const int64_t r = q / a.S;
-    float g[3], n[3], v[3];
-    fd_normal(a, q, g, n);
-    load3(a.w + 3 * r, v);
-    rows[(u + 15) * RS + col] = n[0];
-    rows[(u + 16) * RS + col] = n[1];
-    rows[(u + 17) * RS + col] = n[2];
-    float e[16];
-    encode3<2, 16>(v[0], v[1], v[2], e);
-#pragma unroll
-    for (int k = 0; k < 15; ++k) rows[(u + 18 + k) * RS + col] = e[k];
-}
+// Sample centres run the colour MLP as well; their tiles are 16 records, so that the backward's eight warps of
+// rows and the cell's weights fit in shared memory and its 156 accumulators in registers.
+constexpr int CT = 16;                 // records per warp tile
+constexpr int CRS = row_stride(CT);
+constexpr int CFW = 8, CBW = 8;        // warps per block, forward and backward
 
-// SDF output layer (16 rows: d, z) of the tile into rows[dst .. dst+15]
-__device__ __forceinline__ void output_layer(const float *To, const float *bo, float *rows, int src, int dst) {
-    float acc[2][4];
-    const int o0 = (threadIdx.x >> 5) * 2;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        acc[0][j] = bo[o0];
-        acc[1][j] = bo[o0 + 1];
-    }
-    mm16<32>(To, rows + src * RS, acc);
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-        *reinterpret_cast<float4 *>(rows + (dst + o0 + i) * RS + r0_t()) =
-            make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-}
-
-// colour hidden layer: rows[dst] = relu(C0 rows[u] + c0)
+// what the SDF layers of WW lack: the output layer's T_o[k][16] and biases, the colour layers C0[i][o] (rows
+// past 33 zero) and C1[c][k], and for the backward W_o[o][k] and C0[o][i]
 template <int H>
-__device__ __forceinline__ void colour_hidden(const float *sw, float *rows, int u, int dst) {
+struct WC {
+    static constexpr int To = WW<H>::END, bo = To + 512, C0 = bo + 16, c0 = C0 + 36 * WTS, C1 = c0 + 32, c1 = C1 + 96;
+    static constexpr int FEND = c1 + 4, Wo = FEND, Cr = Wo + 512, END = Cr + 32 * WTS;
+};
+template <int H, bool BACKWARD>
+__device__ __forceinline__ void load_centre_cell(const float *__restrict__ cw, float *sw, int nt) {
     using L = WL<H>;
-    float acc[4][4];
-    init_bias(sw + L::c0, acc);
-    mm32<33, 32>(sw + L::C0t, rows + u * RS, acc);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaxf(acc[i][j], 0.f);
-    store_rows(rows, dst, acc);
-}
-
-// colour logits of record column col from the hidden rows
-template <int H>
-__device__ __forceinline__ void colour_logits(const float *sw, const float *rows, int hc, int col, float (&lg)[3]) {
-    using L = WL<H>;
-    lg[0] = sw[L::c1];
-    lg[1] = sw[L::c1 + 1];
-    lg[2] = sw[L::c1 + 2];
-#pragma unroll 8
-    for (int k = 0; k < 32; ++k) {
-        const float4 w = *reinterpret_cast<const float4 *>(sw + L::C1t + 4 * k);
-        const float h = rows[(hc + k) * RS + col];
-        lg[0] = fmaf(w.x, h, lg[0]);
-        lg[1] = fmaf(w.y, h, lg[1]);
-        lg[2] = fmaf(w.z, h, lg[2]);
-    }
-}
-
-template <int H>
-__global__ void __launch_bounds__(TPB, 2) k_tile_centre_fwd(TrainArgs a) {
-    using L = WL<H>;
-    using R = RL<H>;
-    extern __shared__ float4 smem4[];
-    float *rows = reinterpret_cast<float *>(smem4);
-    float *sw = rows + R::FC_ROWS * RS;
-    __shared__ long long s_q[TILE];
+    using S = WC<H>;
     const int tid = threadIdx.x;
+    load_cell<H, BACKWARD>(cw, sw, nt);
+    for (int j = tid; j < 512; j += nt) {
+        const float v = __ldg(cw + L::cWo + j);
+        sw[S::To + (j & 31) * 16 + (j >> 5)] = v;
+        if (BACKWARD) sw[S::Wo + j] = v;
+    }
+    for (int j = tid; j < 33 * 32; j += nt) {
+        const float v = __ldg(cw + L::cC0 + j);
+        const int o = j / 33, i = j - 33 * o;
+        sw[S::C0 + i * WTS + o] = v;
+        if (BACKWARD) sw[S::Cr + o * WTS + i] = v;
+    }
+    for (int j = tid; j < 3 * WTS; j += nt) sw[S::C0 + 33 * WTS + j] = 0.f;
+    if (tid < 16) sw[S::bo + tid] = __ldg(cw + L::cbo + tid);
+    if (tid < 32) sw[S::c0 + tid] = __ldg(cw + L::cc0 + tid);
+    if (tid < 96) sw[S::C1 + tid] = __ldg(cw + L::cC1 + tid);
+    if (tid < 3) sw[S::c1 + tid] = __ldg(cw + L::cc1 + tid);
+}
+
+// rows of a warp: the encoding and A_1 .. A_H (32 each), the output row d, the colour inputs U (z, n, gamma(v),
+// three zero rows), the upstream of d, the colour hidden layer -- whose rows 0 .. 14 become z's deltas
+// (forward alone: one buffer, a layer overwrites its input)
+template <int H, bool KEEP>
+struct CR {
+    __host__ __device__ static constexpr int A(int l) { return KEEP ? 32 * l : 0; }
+    static constexpr int Ud = KEEP ? 32 * (H + 1) : 32, U = Ud + 1, Dout = U + 36, Hc = Dout + 1, Dc = Hc + 32, ROWS = Dc + 3;
+    static constexpr int GRAD = (WL<H>::cc1 + 3 + 3) / 4 * 4;  // a warp's gradient is put in its rows at the end
+    static constexpr int FLOATS = ROWS * CRS > GRAD ? ROWS * CRS : GRAD;
+};
+
+// A tile forward: lane j and lane j + 16 share record j (q < 0: padding).  Leaves the activations, d and z, the
+// colour inputs and the colour hidden layer in the rows; returns the colour logits in lanes 0 .. 15.
+template <int H, bool KEEP>
+__device__ __forceinline__ void centre_tile(const TrainArgs &a, const float *sw, float *rows, int lane, float4 r,
+                                            long long q, float (&lg)[3]) {
+    using W = WW<H>;
+    using S = WC<H>;
+    using R = CR<H, KEEP>;
+    const int j = lane & 15, h = lane >> 4;
+    {  // Eq. 1: half 0 x and frequencies 0, 1, half 1 frequencies 2, 3; the colour inputs n and gamma(v)
+        const float p[3] = {r.x, r.y, r.z};
+        if (h == 0) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) rows[c * CRS + j] = p[c];
+            if (!KEEP) rows[27 * CRS + j] = 0.f;
+            float n[3] = {0.f, 0.f, 0.f}, g[3];
+            if (q >= 0) fd_normal(a, q, g, n);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) rows[(R::U + 15 + c) * CRS + j] = n[c];
+        } else {
+            float v[3] = {0.f, 0.f, 0.f}, e[16];
+            if (q >= 0) load3(a.w + 3 * (q / a.S), v);
+            encode3<2, 16>(v[0], v[1], v[2], e);
+#pragma unroll
+            for (int k = 0; k < 15; ++k) rows[(R::U + 18 + k) * CRS + j] = e[k];
+        }
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk) {
+            const int k = 2 * h + kk;
+            const float f = (float)(1 << k);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float sn, cs;
+                sincospif(f * p[c], &sn, &cs);
+                rows[(3 + 6 * k + c) * CRS + j] = sn;
+                rows[(6 + 6 * k + c) * CRS + j] = cs;
+            }
+        }
+    }
+    __syncwarp();
+    auto act = [&](float v, int, int) { return softplus(v, a.beta, a.inv_beta); };
+    TileMap<32, CT> m(lane);
+#pragma unroll
+    for (int l = 0; l < H; ++l) {
+        m.bias_shared(sw + W::b(l));
+        if (l == 0) m.template mm_shared<28>(sw + W::T(0), WTS, rows, CRS);
+        else m.template mm_shared<32>(sw + W::T(l), WTS, rows + R::A(l) * CRS, CRS);
+        if (!KEEP) __syncwarp();
+        m.store(rows + R::A(l + 1) * CRS, CRS, act);
+        __syncwarp();
+    }
+    {  // the 16 outputs [d, z]: lane (h, o) output o of records 8 h .. 8 h + 7
+        const float *X = rows + R::A(H) * CRS + 8 * h;
+        float out[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) out[i] = sw[S::bo + j];
+#pragma unroll 4
+        for (int k = 0; k < 32; ++k) {
+            const float w = sw[S::To + k * 16 + j];
+            const float4 x = *reinterpret_cast<const float4 *>(X + k * CRS),
+                         y = *reinterpret_cast<const float4 *>(X + k * CRS + 4);
+            const float xa[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int i = 0; i < 8; ++i) out[i] = fmaf(w, xa[i], out[i]);
+        }
+        float *o = rows + (R::Ud + j) * CRS + 8 * h;  // d, then z in U's rows 0 .. 14
+        *reinterpret_cast<float4 *>(o) = make_float4(out[0], out[1], out[2], out[3]);
+        *reinterpret_cast<float4 *>(o + 4) = make_float4(out[4], out[5], out[6], out[7]);
+    }
+    __syncwarp();
+    m.bias_shared(sw + S::c0);
+    m.template mm_shared<36>(sw + S::C0, WTS, rows + R::U * CRS, CRS);
+    m.store(rows + R::Hc * CRS, CRS, [](float v, int, int) { return fmaxf(v, 0.f); });
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < 3; ++c) lg[c] = sw[S::c1 + c];
+    if (h == 0) {
+#pragma unroll 8
+        for (int k = 0; k < 32; ++k) {
+            const float x = rows[(R::Hc + k) * CRS + j];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) lg[c] = fmaf(sw[S::C1 + 32 * c + k], x, lg[c]);
+        }
+    }
+}
+
+// the rows no tile writes and every tile reads: inputs past the encoding, colour inputs past 33
+template <class R>
+__device__ __forceinline__ void centre_zero_rows(float *rows, int lane) {
+    for (int i = lane; i < 5 * CRS; i += 32) rows[27 * CRS + i] = 0.f;
+    for (int i = lane; i < 3 * CRS; i += 32) rows[(R::U + 33) * CRS + i] = 0.f;
+}
+
+template <int H>
+__global__ void __launch_bounds__(32 * CFW, 2) k_warp_centre_fwd(TrainArgs a) {
+    using S = WC<H>;
+    using R = CR<H, false>;
+    extern __shared__ float4 smem4[];
+    float *sw = reinterpret_cast<float *>(smem4);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float *rows = sw + S::FEND + warp * R::ROWS * CRS;
     const int k0 = a.NC, k1 = 2 * a.NC;
     const int64_t nfd = 6 * (a.B * a.S + a.M);
     const int c0 = a.chunk_off[k0], total = a.chunk_off[k1] - c0;
-    constexpr int last = (H % 2 == 1) ? R::P : R::Q;
-    for (int i = tid; i < R::FC_ROWS * RS; i += TPB) rows[i] = 0.f;
-    __syncthreads();
-    if (tid < TILE) rows[(R::FU + 33) * RS + tid] = 1.f;
+    centre_zero_rows<R>(rows, lane);
     for (int ci = blockIdx.x; ci < total; ci += gridDim.x) {
         const int key = chunk_key(a.chunk_off, k0, k1, c0 + ci);
         const int j = c0 + ci - a.chunk_off[key];
         const int beg = a.off[key] + j * CHUNK, end = min(beg + CHUNK, a.off[key + 1]);
         __syncthreads();
-        load_slots<H>(a.params + (int64_t)(key - a.NC) * a.p_cell, sw, 0, L::FC);
-        for (int tb = beg; tb < end; tb += TILE) {
-            {
-                const int col = tid & (TILE - 1), i = tb + col;
-                float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-                long long q = -1;
-                if (i < end) {
-                    r = a.sorted[i];
-                    q = (long long)__float_as_int(r.w) - nfd;
-                }
-                encode_half(rows, R::A0, col, tid >> 7, r.x, r.y, r.z);
-                if (tid < TILE) {
-                    s_q[tid] = q;
-                    if (q >= 0) centre_inputs(a, rows, R::FU, tid, q);
-                }
+        load_centre_cell<H, false>(a.params + (int64_t)(key - a.NC) * a.p_cell, sw, 32 * CFW);
+        __syncthreads();
+        for (int tb = beg + CT * warp; tb < end; tb += CT * CFW) {
+            const int i = tb + (lane & 15);
+            float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+            long long q = -1;
+            if (i < end) {
+                r = a.sorted[i];
+                q = (long long)__float_as_int(r.w) - nfd;
             }
-            __syncthreads();
-            hidden_layer<27>(sw + L::T0, sw + L::b0, rows, R::A0, R::P, a.beta, a.inv_beta);
-#pragma unroll
-            for (int l = 1; l < H; ++l) {
-                __syncthreads();
-                hidden_layer<32>(sw + L::Tl(l), sw + L::bl(l), rows, (l % 2) ? R::P : R::Q, (l % 2) ? R::Q : R::P,
-                                 a.beta, a.inv_beta);
-            }
-            __syncthreads();
-            output_layer(sw + L::To, sw + L::bo, rows, last, R::FUd);  // d, then z into U rows 0..14
-            __syncthreads();
-            colour_hidden<H>(sw, rows, R::FU, R::FHc);
-            __syncthreads();
-            if (tid < TILE && s_q[tid] >= 0) {
-                const long long q = s_q[tid];
-                float lg[3];
-                colour_logits<H>(sw, rows, R::FHc, tid, lg);
-                a.d_c[q] = rows[R::FUd * RS + tid];
+            float lg[3];
+            centre_tile<H, false>(a, sw, rows, lane, r, q, lg);
+            if (lane < 16 && q >= 0) {
+                a.d_c[q] = rows[R::Ud * CRS + lane];
                 a.rgb_c[3 * q] = sigm(lg[0]);
                 a.rgb_c[3 * q + 1] = sigm(lg[1]);
                 a.rgb_c[3 * q + 2] = sigm(lg[2]);
             }
+            __syncwarp();
         }
     }
 }
 
-// ------------------------------------------------------------------ backward
-// weight-gradient plan: per layer (delta rows, OB, input rows, IB, real outputs, real inputs, canonical
-// W and b offsets); thread block b covers outputs ob + OB jo and inputs ib + IB ji (jo, ji < 4)
-struct GemmLayer {
-    int drow, OB, arow, IB, out_real, in_real, cW, cb;
-};
-
-template <int H, bool CENTRE>
-struct GemmPlan {
-    static constexpr int NL = H + 1 + (CENTRE ? 2 : 0);
-    // the delta rows of layer l's output: difference records keep D_l in place of A_l
-    __host__ __device__ static constexpr int drow(int l) { return CENTRE ? RL<H>::D(l) : RL<H>::A(l); }
-    __host__ __device__ static constexpr int dout() { return CENTRE ? RL<H>::Dout : RL<H>::DoutF; }
-    __device__ static GemmLayer layer(int l) {
-        using L = WL<H>;
-        using R = RL<H>;
-        if (l == 0) return {drow(1), 8, R::A0, 7, 32, 27, L::cW0, L::cb0};
-        if (l < H) return {drow(l + 1), 8, R::A(l), 9, 32, 32, L::cH + (l - 1) * L::HL, L::cH + (l - 1) * L::HL + 1024};
-        if (l == H) return {dout(), CENTRE ? 4 : 1, R::A(H), 9, CENTRE ? 16 : 1, 32, L::cWo, L::cbo};
-        if (l == H + 1) return {R::Dh, 8, R::U, 9, 32, 33, L::cC0, L::cc0};
-        return {R::Dc, 1, R::Hc, 9, 3, 32, L::cC1, L::cc1};
-    }
-    __host__ __device__ static constexpr int blocks() { return 56 + 72 * (H - 1) + (CENTRE ? 36 + 72 + 9 : 9); }
-    static constexpr int NB = (blocks() + TPB - 1) / TPB;
-};
-
-struct Blk {
-    int drow, OB, arow, IB, out_real, in_real, cW, cb, ob, ib, layer;
-};
-
-template <class Plan>
-__device__ __forceinline__ Blk block_of(int b) {
-    Blk k{};
-    k.drow = -1;
-    if (b >= Plan::blocks()) return k;
+// acc[i][j] += sum over the tile's records of D[og + 4 i] A[ig + 8 j], i < NI
+template <int NI>
+__device__ __forceinline__ void grad_tile16(const float *D, const float *A, float (&acc)[NI][4], int lane) {
+    const float *d = D + (lane >> 3) * CRS, *x = A + (lane & 7) * CRS;
 #pragma unroll 1
-    for (int l = 0; l < Plan::NL; ++l) {
-        const GemmLayer G = Plan::layer(l);
-        const int n = G.OB * G.IB;
-        if (b < n) {
-            k.layer = l;
-            k.drow = G.drow;
-            k.OB = G.OB;
-            k.arow = G.arow;
-            k.IB = G.IB;
-            k.out_real = G.out_real;
-            k.in_real = G.in_real;
-            k.cW = G.cW;
-            k.cb = G.cb;
-            if (G.IB == 9) {
-                // eight consecutive lanes (one shared-memory phase of a 16-byte load) take input rows
-                // ib = 0..7 of one output group, so their rows fall in distinct bank groups; the
-                // ib = 8 blocks follow, one per output group
-                if (b < 8 * G.OB) {
-                    k.ob = b >> 3;
-                    k.ib = b & 7;
-                } else {
-                    k.ob = b - 8 * G.OB;
-                    k.ib = 8;
-                }
-            } else {
-                k.ob = b / G.IB;
-                k.ib = b - k.ob * G.IB;
+    for (int r = 0; r < CT; r += 4) {
+        float4 xv[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) xv[j] = *reinterpret_cast<const float4 *>(x + 8 * j * CRS + r);
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            const float4 dv = *reinterpret_cast<const float4 *>(d + 4 * i * CRS + r);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float s = acc[i][j];
+                s = fmaf(dv.x, xv[j].x, s);
+                s = fmaf(dv.y, xv[j].y, s);
+                s = fmaf(dv.z, xv[j].z, s);
+                s = fmaf(dv.w, xv[j].w, s);
+                acc[i][j] = s;
             }
-            return k;
         }
-        b -= n;
-    }
-    return k;
-}
-
-// layer >= 0: only the blocks of that plan layer
-template <class Plan>
-__device__ __forceinline__ void grad_tile(const float *rows, int b, float (&acc)[16], int layer = -1) {
-    const Blk k = block_of<Plan>(b);
-    if (k.drow < 0 || (layer >= 0 && k.layer != layer)) return;
-    const float *D = rows + (k.drow + k.ob) * RS;
-    const float *A = rows + (k.arow + k.ib) * RS;
-    const int sd = k.OB * RS, sa = k.IB * RS;
-#pragma unroll 2
-    for (int r = 0; r < TILE; r += 4) {
-        float4 dv[4], av[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            dv[q] = *reinterpret_cast<const float4 *>(D + q * sd + r);
-            av[q] = *reinterpret_cast<const float4 *>(A + q * sa + r);
-        }
-#pragma unroll
-        for (int jo = 0; jo < 4; ++jo)
-#pragma unroll
-            for (int ji = 0; ji < 4; ++ji) {
-                float s = acc[jo * 4 + ji];
-                s = fmaf(dv[jo].x, av[ji].x, s);
-                s = fmaf(dv[jo].y, av[ji].y, s);
-                s = fmaf(dv[jo].z, av[ji].z, s);
-                s = fmaf(dv[jo].w, av[ji].w, s);
-                acc[jo * 4 + ji] = s;
-            }
     }
 }
-
-template <class Plan>
-__device__ __forceinline__ void flush_grad(float *gcell, int b, float (&acc)[16]) {
-    const Blk k = block_of<Plan>(b);
-    if (k.drow < 0) return;
+// sum over the tile's records of x times y (y NULL: 1), rows of CT records
+__device__ __forceinline__ float row_dot16(const float *x, const float *y) {
+    float s = 0.f;
 #pragma unroll
-    for (int jo = 0; jo < 4; ++jo)
-#pragma unroll
-        for (int ji = 0; ji < 4; ++ji) {
-            const int o = k.ob + k.OB * jo, i = k.ib + k.IB * ji;
-            const float v = acc[jo * 4 + ji];
-            acc[jo * 4 + ji] = 0.f;
-            if (v == 0.f || o >= k.out_real || i > k.in_real) continue;
-            atomicAdd(gcell + (i < k.in_real ? k.cW + o * k.in_real + i : k.cb + o), v);
-        }
+    for (int r = 0; r < CT; r += 4) {
+        const float4 u = *reinterpret_cast<const float4 *>(x + r);
+        const float4 v = y ? *reinterpret_cast<const float4 *>(y + r) : make_float4(1.f, 1.f, 1.f, 1.f);
+        s = fmaf(u.x, v.x, s);
+        s = fmaf(u.y, v.y, s);
+        s = fmaf(u.z, v.z, s);
+        s = fmaf(u.w, v.w, s);
+    }
+    return s;
 }
 
-// D_l = (W_l^T D_{l+1}) . softplus'(A_l) for l = H-1 .. 1 (D_H already in its rows)
+// Sample centres backward: the tile recomputed forward, the colour MLP's deltas, then the SDF's with upstream on d
+// and z; writes the difference points' upstream.  Weight gradients stay in registers over the chunk as in
+// k_warp_fd_backward: lane (og, ig) owns outputs og + 4 i and inputs ig + 8 j of every layer.
 template <int H>
-__device__ __forceinline__ void hidden_backward(const float *sw, float *rows, float beta) {
+__global__ void __launch_bounds__(32 * CBW, 1) k_warp_centre_backward(TrainArgs a) {
     using L = WL<H>;
-    using R = RL<H>;
-#pragma unroll
-    for (int l = H - 1; l >= 1; --l) {
-        __syncthreads();
-        float acc[4][4], act[4][4];
-        zero(acc);
-        mm32<32, 32>(sw + L::Wr(l), rows + R::D(l + 1) * RS, acc);
-        load_rows(rows, R::A(l), act);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] *= dsoftplus_act(act[i][j], beta);
-        store_rows(rows, R::D(l), acc);
-    }
-}
-
-// CENTRE: sample-centre records (colour MLP + SDF with upstream on d and z; writes the difference
-// records' upstream).  Otherwise: difference records (SDF with upstream on d only).
-template <int H, bool CENTRE>
-__global__ void __launch_bounds__(TPB, CENTRE ? 1 : 2) k_tile_backward(TrainArgs a) {
-    using L = WL<H>;
-    using R = RL<H>;
-    using Plan = GemmPlan<H, CENTRE>;
-    constexpr int NROWS = CENTRE ? R::C_ROWS : R::FDI_ROWS;
+    using W = WW<H>;
+    using S = WC<H>;
+    using R = CR<H, true>;
+    constexpr int NT = 32 * CBW;
     extern __shared__ float4 smem4[];
-    float *rows = reinterpret_cast<float *>(smem4);
-    float *sw = rows + NROWS * RS;
-    __shared__ long long s_q[TILE];
-    const int tid = threadIdx.x;
-    for (int i = tid; i < NROWS * RS; i += TPB) rows[i] = 0.f;
-    __syncthreads();
-    if (tid < TILE) {
-        rows[(R::A0 + 27) * RS + tid] = 1.f;
-        for (int l = 1; l <= H; ++l) rows[(R::A(l) + 32) * RS + tid] = 1.f;
-        if (CENTRE) {
-            rows[(R::U + 33) * RS + tid] = 1.f;
-            rows[(R::Hc + 32) * RS + tid] = 1.f;
-        }
-    }
-    float acc[Plan::NB][16];
-#pragma unroll
-    for (int k = 0; k < Plan::NB; ++k)
-#pragma unroll
-        for (int e = 0; e < 16; ++e) acc[k][e] = 0.f;
-    const int k0 = CENTRE ? a.NC : 0, k1 = CENTRE ? 2 * a.NC : a.NC;
+    float *sw = reinterpret_cast<float *>(smem4);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float *all = sw + S::END, *rows = all + warp * R::FLOATS;
+    const int k0 = a.NC, k1 = 2 * a.NC;
     const int64_t nfd = 6 * (a.B * a.S + a.M);
     const int c0 = a.chunk_off[k0], total = a.chunk_off[k1] - c0;
     const float inv2h = 1.f / (2.f * a.h);
     for (int ci = blockIdx.x; ci < total; ci += gridDim.x) {
         const int key = chunk_key(a.chunk_off, k0, k1, c0 + ci);
         const int cell = key - k0;
-        const int j = c0 + ci - a.chunk_off[key];
-        const int beg = a.off[key] + j * CHUNK, end = min(beg + CHUNK, a.off[key + 1]);
-        const float *cw = a.params + (int64_t)cell * a.p_cell;
+        const int jc = c0 + ci - a.chunk_off[key];
+        const int beg = a.off[key] + jc * CHUNK, end = min(beg + CHUNK, a.off[key + 1]);
         __syncthreads();
-        load_slots<H>(cw, sw, 0, L::FS);
-        if (CENTRE) load_slots<H>(cw, sw, L::FS, L::END);
-        else load_slots<H>(cw, sw, L::FC, L::BS);
-        for (int tb = beg; tb < end; tb += TILE) {
-            // records: encoding, and the upstream of d (difference points) or the colour inputs (centres)
+        load_centre_cell<H, true>(a.params + (int64_t)cell * a.p_cell, sw, NT);
+        centre_zero_rows<R>(rows, lane);
+        __syncthreads();
+        float dw[H][8][4], dwo[4][4], dwc[8][4], db[H], dbo = 0.f, dbc0 = 0.f, dwc32 = 0.f, dc1[3], dbc1[3];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                for (int l = 0; l < H; ++l) dw[l][i][k] = 0.f;
+                dwc[i][k] = 0.f;
+                if (i < 4) dwo[i][k] = 0.f;
+            }
+#pragma unroll
+        for (int l = 0; l < H; ++l) db[l] = 0.f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) dc1[c] = dbc1[c] = 0.f;
+        for (int tb = beg + CT * warp; tb < end; tb += CT * CBW) {
+            const int i = tb + (lane & 15);
+            float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+            long long q = -1;
+            if (i < end) {
+                r = a.sorted[i];
+                q = (long long)__float_as_int(r.w) - nfd;
+            }
+            float lg[3];
+            centre_tile<H, true>(a, sw, rows, lane, r, q, lg);
+            if (lane < 16) {  // logits -> colour delta; the upstream of d
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const float rgb = sigm(lg[c]);
+                    const float dc = q >= 0 ? a.g_rgb[3 * q + c] * rgb * (1.f - rgb) : 0.f;
+                    rows[(R::Dc + c) * CRS + lane] = dc;
+                    dbc1[c] += dc;
+                }
+                rows[R::Dout * CRS + lane] = q >= 0 ? a.g_dc[q] : 0.f;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < 3; ++c) dc1[c] += row_dot16(rows + (R::Hc + lane) * CRS, rows + (R::Dc + c) * CRS);
+            __syncwarp();
+            TileMap<32, CT> m(lane);
+            {  // Dh = (Wc1^T Dc) . [Hc > 0] over Hc
+                float *own = rows + R::Hc * CRS;
+                const float *dc = rows + R::Dc * CRS;
+                m.zero();
+                m.store(own, CRS, [&](float, int u, int s) {
+                    const float v = fmaf(sw[S::C1 + u], dc[s], fmaf(sw[S::C1 + 32 + u], dc[CRS + s],
+                                                                   sw[S::C1 + 64 + u] * dc[2 * CRS + s]));
+                    return own[u * CRS + s] > 0.f ? v : 0.f;
+                });
+            }
+            __syncwarp();
+            grad_tile16<8>(rows + R::Hc * CRS, rows + R::U * CRS, dwc, lane);
+            dwc32 += row_dot16(rows + (R::Hc + lane) * CRS, rows + (R::U + 32) * CRS);
+            dbc0 += row_dot16(rows + (R::Hc + lane) * CRS, nullptr);
+            // input deltas over Dh: rows 0 .. 14 z's, 15 .. 17 the normal's
+            m.zero();
+            m.template mm_shared<32>(sw + S::Cr, WTS, rows + R::Hc * CRS, CRS);
+            __syncwarp();
+            m.store(rows + R::Hc * CRS, CRS, [](float v, int, int) { return v; });
+            __syncwarp();
+            if (lane < 16 && q >= 0) {  // the normal's delta to the difference records
+                float g[3], n[3];
+                const float gn = fd_normal(a, q, g, n);
+                const float gx = rows[(R::Hc + 15) * CRS + lane], gy = rows[(R::Hc + 16) * CRS + lane],
+                            gz = rows[(R::Hc + 17) * CRS + lane];
+                const float nd = n[0] * gx + n[1] * gy + n[2] * gz;
+                const float ig = gn > 0.f ? inv2h / gn : 0.f;
+                const float dg[3] = {(gx - n[0] * nd) * ig, (gy - n[1] * nd) * ig, (gz - n[2] * nd) * ig};
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    a.g_fd[6 * q + 2 * k] = dg[k];
+                    a.g_fd[6 * q + 2 * k + 1] = -dg[k];
+                }
+            }
+            // output layer: its gradient, then D_H = (Wo^T Dout) . softplus'(A_H) over A_H
+            grad_tile16<4>(rows + R::Dout * CRS, rows + R::A(H) * CRS, dwo, lane);
+            if (lane < 16) dbo += row_dot16(rows + (R::Dout + lane) * CRS, nullptr);
             {
-                const int col = tid & (TILE - 1), i = tb + col;
-                float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-                long long q = -1;
-                if (i < end) {
-                    r = a.sorted[i];
-                    q = (long long)__float_as_int(r.w) - (CENTRE ? nfd : 0);
-                }
-                encode_half(rows, R::A0, col, tid >> 7, r.x, r.y, r.z);
-                if (tid < TILE) {
-                    s_q[tid] = q;
-                    if (CENTRE) {
-                        if (q >= 0) centre_inputs(a, rows, R::U, tid, q);
-                    } else {
-                        rows[R::DoutF * RS + tid] = q >= 0 ? a.g_fd[q] : 0.f;
-                    }
-                }
+                float *own = rows + R::A(H) * CRS;
+                m.zero();
+                m.template mm_shared<16>(sw + S::Wo, 32, rows + R::Dout * CRS, CRS);
+                __syncwarp();
+                m.store(own, CRS, [&](float v, int u, int s) { return v * dsoftplus_act(own[u * CRS + s], a.beta); });
             }
-            __syncthreads();
-            hidden_layer<27>(sw + L::T0, sw + L::b0, rows, R::A0, R::A(1), a.beta, a.inv_beta);
+            __syncwarp();
 #pragma unroll
-            for (int l = 1; l < H; ++l) {
-                __syncthreads();
-                hidden_layer<32>(sw + L::Tl(l), sw + L::bl(l), rows, R::A(l), R::A(l + 1), a.beta, a.inv_beta);
+            for (int l = H - 1; l >= 1; --l) {
+                const float *D = rows + R::A(l + 1) * CRS;
+                float *own = rows + R::A(l) * CRS;
+                grad_tile16<8>(D, own, dw[l], lane);
+                db[l] += row_dot16(D + lane * CRS, nullptr);
+                m.zero();
+                m.template mm_shared<32>(sw + W::R(l), 32, D, CRS);
+                __syncwarp();
+                m.store(own, CRS, [&](float v, int u, int s) { return v * dsoftplus_act(own[u * CRS + s], a.beta); });
+                __syncwarp();
             }
-            __syncthreads();
-            if (CENTRE) {
-                output_layer(sw + L::To, sw + L::bo, rows, R::A(H), R::Ud);  // d, then z into U rows 0..14
-                __syncthreads();
-                colour_hidden<H>(sw, rows, R::U, R::Hc);
-                __syncthreads();
-                // logits -> colour delta (rows Dc)
-                if (tid < TILE) {
-                    const long long q = s_q[tid];
-                    float lg[3];
-                    colour_logits<H>(sw, rows, R::Hc, tid, lg);
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        const float rgb = sigm(lg[c]);
-                        rows[(R::Dc + c) * RS + tid] = q >= 0 ? a.g_rgb[3 * q + c] * rgb * (1.f - rgb) : 0.f;
-                    }
-                }
-                __syncthreads();
-                // hidden delta: Dh = (Wc1^T Dc) . [Hc > 0]
-                {
-                    float dh[4][4], hv[4][4];
-                    load_rows(rows, R::Hc, hv);
-                    const int o0 = o0_32(), r0 = r0_t();
-                    float dc[3][4];
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        const float4 x = *reinterpret_cast<const float4 *>(rows + (R::Dc + c) * RS + r0);
-                        dc[c][0] = x.x;
-                        dc[c][1] = x.y;
-                        dc[c][2] = x.z;
-                        dc[c][3] = x.w;
-                    }
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float w0 = sw[L::Wc1 + o0 + i], w1 = sw[L::Wc1 + 32 + o0 + i],
-                                    w2 = sw[L::Wc1 + 64 + o0 + i];
-#pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) {
-                            const float s = fmaf(w0, dc[0][jj], fmaf(w1, dc[1][jj], w2 * dc[2][jj]));
-                            dh[i][jj] = hv[i][jj] > 0.f ? s : 0.f;
-                        }
-                    }
-                    store_rows(rows, R::Dh, dh);
-                }
-                __syncthreads();
-                // input deltas of z and n: gu[i] = sum_o Wc0[o][i] Dh[o]; two threads per record
-                {
-                    const int col = tid & (TILE - 1), half = tid >> 7;
-                    const long long q = s_q[col];
-                    const int i0 = half ? 9 : 0;
-                    float gu[9];
-#pragma unroll
-                    for (int m = 0; m < 9; ++m) gu[m] = 0.f;
-#pragma unroll 4
-                    for (int o = 0; o < 32; ++o) {
-                        const float dh = rows[(R::Dh + o) * RS + col];
-#pragma unroll
-                        for (int m = 0; m < 9; ++m) gu[m] = fmaf(sw[L::Wc0 + o * 36 + i0 + m], dh, gu[m]);
-                    }
-                    // z deltas (+ the d upstream) into Dout; the normal's delta to the difference records
-#pragma unroll
-                    for (int m = 0; m < 9; ++m)
-                        if (i0 + m < 15) rows[(R::Dout + 1 + i0 + m) * RS + col] = gu[m];
-                    if (half == 0) {
-                        rows[R::Dout * RS + col] = q >= 0 ? a.g_dc[q] : 0.f;
-                    } else if (q >= 0) {
-                        float g[3], n[3];
-                        const float gn = fd_normal(a, q, g, n);
-                        const float gx = gu[6], gy = gu[7], gz = gu[8];  // inputs 15, 16, 17
-                        const float nd = n[0] * gx + n[1] * gy + n[2] * gz;
-                        const float ig = gn > 0.f ? inv2h / gn : 0.f;
-                        const float dg[3] = {(gx - n[0] * nd) * ig, (gy - n[1] * nd) * ig, (gz - n[2] * nd) * ig};
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) {
-                            a.g_fd[6 * q + 2 * k] = dg[k];
-                            a.g_fd[6 * q + 2 * k + 1] = -dg[k];
-                        }
-                    }
-                }
-                __syncthreads();
-                // D_H = (Wo^T Dout) . softplus'(A_H)
-                {
-                    float acc2[4][4], act[4][4];
-                    zero(acc2);
-                    mm32<16, 32>(sw + L::Wo, rows + R::Dout * RS, acc2);
-                    load_rows(rows, R::A(H), act);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) acc2[i][jj] *= dsoftplus_act(act[i][jj], a.beta);
-                    store_rows(rows, R::D(H), acc2);
-                }
-                hidden_backward<H>(sw, rows, a.beta);
-                __syncthreads();
-#pragma unroll
-                for (int k = 0; k < Plan::NB; ++k) grad_tile<Plan>(rows, tid + k * TPB, acc[k]);
-                __syncthreads();
-            } else {
-                // Difference records, deltas in place of the activations (so two blocks fit per SM): each
-                // layer's weight gradient is taken while its input activations are still in their rows.
-                // Output layer first (Dout x A_H), then D_H = Wo[0] g . softplus'(A_H) over A_H.
-#pragma unroll
-                for (int k = 0; k < Plan::NB; ++k) grad_tile<Plan>(rows, tid + k * TPB, acc[k], H);
-                __syncthreads();
-                {
-                    float act[4][4], dd[4][4];
-                    load_rows(rows, R::A(H), act);
-                    const float4 g4 = *reinterpret_cast<const float4 *>(rows + R::DoutF * RS + r0_t());
-                    const float g[4] = {g4.x, g4.y, g4.z, g4.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float w = sw[L::Wo + o0_32() + i];
-#pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) dd[i][jj] = w * g[jj] * dsoftplus_act(act[i][jj], a.beta);
-                    }
-                    store_rows(rows, R::A(H), dd);  // each thread reads and writes only its own block
-                }
-                // hidden layer l: its weight gradient (D_{l+1} x A_l), then D_l over A_l
-#pragma unroll
-                for (int l = H - 1; l >= 1; --l) {
-                    __syncthreads();
-#pragma unroll
-                    for (int k = 0; k < Plan::NB; ++k) grad_tile<Plan>(rows, tid + k * TPB, acc[k], l);
-                    __syncthreads();
-                    float dacc[4][4], act[4][4];
-                    zero(dacc);
-                    mm32<32, 32>(sw + L::Wr(l), rows + R::A(l + 1) * RS, dacc);
-                    load_rows(rows, R::A(l), act);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) dacc[i][jj] *= dsoftplus_act(act[i][jj], a.beta);
-                    store_rows(rows, R::A(l), dacc);
-                }
-                __syncthreads();
-#pragma unroll
-                for (int k = 0; k < Plan::NB; ++k) grad_tile<Plan>(rows, tid + k * TPB, acc[k], 0);
-                __syncthreads();
-            }
+            grad_tile16<8>(rows + R::A(1) * CRS, rows, dw[0], lane);
+            db[0] += row_dot16(rows + (R::A(1) + lane) * CRS, nullptr);
+            __syncwarp();
         }
-        float *gcell = a.grad + (int64_t)cell * a.p_cell;
+        // the chunk's gradient: each warp's in its rows, canonical order; then summed over the warps
+        const int og = lane >> 3, ig = lane & 7;
 #pragma unroll
-        for (int k = 0; k < Plan::NB; ++k) flush_grad<Plan>(gcell, tid + k * TPB, acc[k]);
+        for (int l = 0; l < H; ++l) {
+            const int K = l == 0 ? 27 : 32, cW = l == 0 ? L::cW0 : L::cH + (l - 1) * L::HL;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (ig + 8 * k < K) rows[cW + (og + 4 * i) * K + ig + 8 * k] = dw[l][i][k];
+            rows[cW + 32 * K + lane] = db[l];
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (i < 4) rows[L::cWo + (og + 4 * i) * 32 + ig + 8 * k] = dwo[i][k];
+                rows[L::cC0 + (og + 4 * i) * 33 + ig + 8 * k] = dwc[i][k];
+            }
+        if (lane < 16) rows[L::cbo + lane] = dbo;
+        rows[L::cC0 + lane * 33 + 32] = dwc32;
+        rows[L::cc0 + lane] = dbc0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            rows[L::cC1 + 32 * c + lane] = dc1[c];
+            float v = dbc1[c];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) rows[L::cc1 + c] = v;
+        }
+        __syncthreads();
+        const int nw = min(CBW, (end - beg + CT - 1) / CT);  // warps that had a tile
+        float *gcell = a.grad + (int64_t)cell * a.p_cell;
+        for (int e = tid; e < L::cc1 + 3; e += NT) {
+            float v = 0.f;
+            for (int w = 0; w < nw; ++w) v += all[w * R::FLOATS + e];
+            if (v != 0.f) atomicAdd(gcell + e, v);
+        }
     }
 }
 
 // ------------------------------------------------------------------ launchers
-template <int H>
-size_t eval_smem() { return ((size_t)RL<H>::F_ROWS * RS + WL<H>::FS) * sizeof(float); }
-template <int H>
-size_t centre_fwd_smem() { return ((size_t)RL<H>::FC_ROWS * RS + WL<H>::FC) * sizeof(float); }
-template <int H>
-size_t backward_smem(bool centre) {
-    return ((size_t)(centre ? RL<H>::C_ROWS : RL<H>::FDI_ROWS) * RS + (centre ? WL<H>::END : WL<H>::BS)) *
-           sizeof(float);
-}
-
 template <class F>
 cudaError_t set_smem(F f, size_t bytes) {
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -787,29 +721,37 @@ cudaError_t set_smem(F f, size_t bytes) {
 
 template <int H>
 cudaError_t eval_d_h(const TrainArgs &a, int k0, int k1, float *out, int64_t chunks, int sm_count, cudaStream_t s) {
-    const size_t sm = eval_smem<H>();
-    cudaError_t e = set_smem(k_tile_eval_d<H>, sm);
+    const size_t sm = (WW<H>::FEND + FW * 32 * WRS) * sizeof(float);
+    cudaError_t e = set_smem(k_warp_eval_d<H>, sm);
     if (e != cudaSuccess) return e;
-    k_tile_eval_d<H><<<grid_for(sm_count, 3, chunks), TPB, sm, s>>>(a, k0, k1, out);
+    k_warp_eval_d<H><<<grid_for(sm_count, 2, chunks), 32 * FW, sm, s>>>(a, k0, k1, out);
     return cudaGetLastError();
 }
 
 template <int H>
 cudaError_t centre_fwd_h(const TrainArgs &a, int64_t chunks, int sm_count, cudaStream_t s) {
-    const size_t sm = centre_fwd_smem<H>();
-    cudaError_t e = set_smem(k_tile_centre_fwd<H>, sm);
+    const size_t sm = (WC<H>::FEND + CFW * CR<H, false>::ROWS * CRS) * sizeof(float);
+    cudaError_t e = set_smem(k_warp_centre_fwd<H>, sm);
     if (e != cudaSuccess) return e;
-    k_tile_centre_fwd<H><<<grid_for(sm_count, 2, chunks), TPB, sm, s>>>(a);
+    k_warp_centre_fwd<H><<<grid_for(sm_count, 2, chunks), 32 * CFW, sm, s>>>(a);
     return cudaGetLastError();
 }
 
-template <int H, bool CENTRE>
-cudaError_t backward_h(const TrainArgs &a, int64_t chunks, int sm_count, cudaStream_t s) {
-    const size_t sm = backward_smem<H>(CENTRE);
-    cudaError_t e = set_smem(k_tile_backward<H, CENTRE>, sm);
+template <int H>
+cudaError_t centre_backward_h(const TrainArgs &a, int64_t chunks, int sm_count, cudaStream_t s) {
+    const size_t sm = (WC<H>::END + CBW * CR<H, true>::FLOATS) * sizeof(float);
+    cudaError_t e = set_smem(k_warp_centre_backward<H>, sm);
     if (e != cudaSuccess) return e;
-    // difference records hold their deltas in place of the activations: two blocks fit per SM
-    k_tile_backward<H, CENTRE><<<grid_for(sm_count, CENTRE ? 1 : 2, chunks), TPB, sm, s>>>(a);
+    k_warp_centre_backward<H><<<grid_for(sm_count, 1, chunks), 32 * CBW, sm, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <int H>
+cudaError_t fd_backward_h(const TrainArgs &a, int64_t chunks, int sm_count, cudaStream_t s) {
+    const size_t sm = (WW<H>::END + BW * WRows<H>::ROWS * WRS) * sizeof(float);
+    cudaError_t e = set_smem(k_warp_fd_backward<H>, sm);
+    if (e != cudaSuccess) return e;
+    k_warp_fd_backward<H><<<grid_for(sm_count, 2, chunks), 32 * BW, sm, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -835,13 +777,13 @@ cudaError_t train_centre_forward(const TrainArgs &a, int sm_count, cudaStream_t 
 }
 
 cudaError_t train_centre_backward(const TrainArgs &a, int sm_count, cudaStream_t s) {
-    return a.H == 3 ? backward_h<3, true>(a, centre_chunks(a), sm_count, s)
-                    : backward_h<2, true>(a, centre_chunks(a), sm_count, s);
+    return a.H == 3 ? centre_backward_h<3>(a, centre_chunks(a), sm_count, s)
+                    : centre_backward_h<2>(a, centre_chunks(a), sm_count, s);
 }
 
 cudaError_t train_fd_backward(const TrainArgs &a, int sm_count, cudaStream_t s) {
-    return a.H == 3 ? backward_h<3, false>(a, fd_chunks(a), sm_count, s)
-                    : backward_h<2, false>(a, fd_chunks(a), sm_count, s);
+    return a.H == 3 ? fd_backward_h<3>(a, fd_chunks(a), sm_count, s)
+                    : fd_backward_h<2>(a, fd_chunks(a), sm_count, s);
 }
 
 }  // namespace kns

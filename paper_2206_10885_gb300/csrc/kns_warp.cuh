@@ -124,6 +124,47 @@ struct TileMap {
             move<0, 2>();
         }
     }
+    // The same with the weight rows in shared memory (16-byte aligned).
+    template <int K>
+    __device__ __forceinline__ void mm_shared(const float *wk, int ws, const float *x, int xs) {
+        const float *xp = x + s0, *wp = wk + u0;
+#pragma unroll 4
+        for (int k = 0; k < K; ++k) {
+            f32x2 t[S / 2];
+            if constexpr (S == 2) {
+                t[0] = *reinterpret_cast<const f32x2 *>(xp + k * xs);
+            } else {
+#pragma unroll
+                for (int j = 0; j < S / 4; ++j) {
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(xp + k * xs + 16 * j);
+                    t[2 * j] = v.x;
+                    t[2 * j + 1] = v.y;
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < NU / 4; ++h) {
+                const float4 v = *reinterpret_cast<const float4 *>(wp + k * ws + 32 * h);
+                const float vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const f32x2 d = f2_pack(vv[i], vv[i]);
+#pragma unroll
+                    for (int j = 0; j < S / 2; ++j) acc[4 * h + i][j] = f2_fma(d, t[j], acc[4 * h + i][j]);
+                }
+            }
+        }
+    }
+    __device__ __forceinline__ void bias_shared(const float *b) {
+#pragma unroll
+        for (int h = 0; h < NU / 4; ++h) {
+            const float4 v = *reinterpret_cast<const float4 *>(b + u0 + 32 * h);
+            const float vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < S / 2; ++j) acc[4 * h + i][j] = f2_pack(vv[i], vv[i]);
+        }
+    }
     // rows[unit][sample] = f(sum, unit, sample)
     template <class F>
     __device__ __forceinline__ void store(float *rows, int xs, F f) const {
