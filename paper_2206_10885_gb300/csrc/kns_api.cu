@@ -27,6 +27,8 @@ struct WaveScratch {
     int *steps_ray = nullptr, *cell_ray = nullptr, *q[2] = {nullptr, nullptr}, *qcell[2] = {nullptr, nullptr};
     int *sorted = nullptr, *hits = nullptr;
     int *cellbuf = nullptr;  // count[2], fill[2], off, tile_off (6 * (nc + 1) ints)
+    int *buckets = nullptr;  // persistent BF16 trace: bucket[2], list[2], taken (kns_kernels.h)
+    int bucket_nc = 0;       // cells they are sized for
     int4 *tiles = nullptr;   // tile descriptors of a round (max_tiles(rays, 2 nc))
     int *pend_r[2] = {nullptr, nullptr};  // per round parity: rays waiting for the occupancy DDA
     float *pend_t[2] = {nullptr, nullptr};
@@ -368,6 +370,7 @@ void free_scratch(WaveScratch &w) {
     cudaFree(w.hits);
     cudaFree(w.cellbuf);
     cudaFree(w.tiles);
+    cudaFree(w.buckets);
     for (int p = 0; p < 2; ++p) {
         cudaFree(w.pend_r[p]);
         cudaFree(w.pend_t[p]);
@@ -1133,7 +1136,26 @@ kns_status render_views_impl(kns_ctx *ctx, const kns_grid *grid, const std::vect
     a.off = w.cellbuf + 4 * (nkeys + 1);
     a.tile_off = w.cellbuf + 5 * (nkeys + 1);
     a.ctrl = w.ctrl;
+    if (cfg.bf16 && cfg.persistent) {
+        const size_t per = (size_t)(2 * kns::kBucket) * nkeys, lists = (size_t)2 * (kns::kBucket / 128) * nkeys;
+        if (w.bucket_nc < nkeys) {  // without them (no memory left) every round is sorted
+            cudaDeviceSynchronize();
+            cudaFree(w.buckets);
+            w.buckets = nullptr;
+            w.bucket_nc = 0;
+            if (cudaMalloc((void **)&w.buckets, sizeof(int) * (per + lists + nkeys)) == cudaSuccess) w.bucket_nc = nkeys;
+            else cudaGetLastError();
+        }
+        if (w.buckets) {
+            for (int p = 0; p < 2; ++p) {
+                a.bucket[p] = w.buckets + p * (per / 2);
+                a.list[p] = w.buckets + per + p * (lists / 2);
+            }
+            a.taken = w.buckets + per + lists;
+        }
+    }
     cudaError_t e = cudaMemcpyAsync(w.d_views, views.data(), sizeof(kns::ViewDev) * nv, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && a.taken) e = cudaMemsetAsync(a.taken, 0, sizeof(int) * (size_t)nkeys, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(w.ctrl, 0, sizeof(kns::WaveCtrl), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(w.cellbuf, 0, sizeof(int) * 4 * (nkeys + 1), s);
     if (e == cudaSuccess) {

@@ -33,6 +33,8 @@ struct WaveCtrl {
     int next_adv;                     // the previous round's pending rays handed out to warps
     int rounds;                       // rounds it ran
     int tail_parity;                  // queue parity of the round it left to the one-warp-per-ray tail
+    int n_list[2];                    // by parity: tiles listed for the round while its samples were queued ...
+    int over[2];                      // ... and whether a cell held more than kBucket samples
     int round_live[512];              // samples queued for each round
     int round_tiles[512];             // tiles of each round (persistent BF16 trace)
     unsigned long long round_end_ns[512];  // global timer at the end of each round
@@ -40,6 +42,8 @@ struct WaveCtrl {
     unsigned long long start_ns;      // global timer at its start
 };
 constexpr int kMaxTraceRounds = 512;
+constexpr int kBucket = 512;            // samples of a cell a sparse round keeps without sorting
+constexpr int kBucketRays = 1 << 16;    // a round of at most this many samples queues its successor in buckets
 
 // One view of a render: its camera, image size, first ray id and output buffers (device, 128 B).
 struct ViewDev {
@@ -90,6 +94,9 @@ struct WaveArgs {
     int *sorted, *hits;
     int *count[2], *fill[2];  // per-cell sample counts and scatter cursors
     int *off, *tile_off;      // NC+1 exclusive scans: samples and tiles per cell
+    // persistent BF16 trace: per parity, kBucket samples of every cell and the round's tiles (cell, number of the
+    // 128 in the cell << 18); per cell, its tiles already taken.  NULL: every round is sorted.
+    int *bucket[2], *list[2], *taken;
     int4 *tiles;              // per tile of the round: key, first sorted sample, samples (max_tiles entries)
     int *pend_r[2];           // per round parity: rays waiting for the occupancy DDA (bit 31: BF16 phase) ...
     float *pend_t[2];         // ... and the position each was last evaluated at

@@ -223,11 +223,30 @@ __device__ __forceinline__ int advance_fast(const GridView &g, const Ray &r, flo
     return cell_of(g, x, y, z);
 }
 
+// As warp_count_cells for the queue of parity p, also putting each ray r into its cell's bucket and a tile on the
+// round's list for every 128 of a cell: a round queued this way needs no sort.
+__device__ __forceinline__ void warp_bucket_cells(const WaveArgs &a, int p, bool pred, int cell, int r) {
+    const unsigned m = __ballot_sync(FULL, pred);
+    if (pred) {
+        const unsigned grp = __match_any_sync(m, cell);
+        const int leader = __ffs(grp) - 1;
+        int rank = 0;
+        if ((int)(threadIdx.x & 31) == leader) rank = atomicAdd(a.count[p] + cell, __popc(grp));
+        rank = __shfl_sync(grp, rank, leader) + __popc(grp & lanemask_lt());
+        if (rank < kBucket) {
+            a.bucket[p][cell * kBucket + rank] = r;
+            if ((rank & 127) == 0) a.list[p][atomicAdd(&a.ctrl->n_list[p], 1)] = cell | (rank >> 7) << 18;
+        } else {
+            a.ctrl->over[p] = 1;
+        }
+    }
+}
+
 // Entry i of the pending list of parity p_in (i < n; every lane of the warp calls it): the ray walks the
 // occupancy DDA from its position to its next occupied voxel (or leaves the grid: a miss), takes the
 // cycle test on the position reached, and joins the queue, counts and live counter of parity p_out.
 __device__ __forceinline__ void advance_pending(const GridView &g, const WaveArgs &a, int p_in, int p_out, int i,
-                                                int n) {
+                                                int n, bool buckets = false) {
     bool emit = false;
     int ncell = -1, r = 0, key = 0;
     if (i < n) {
@@ -264,15 +283,21 @@ __device__ __forceinline__ void advance_pending(const GridView &g, const WaveArg
         a.q[p_out][qp] = r;
         a.qcell[p_out][qp] = key;
     }
-    warp_count_cells(a.count[p_out], emit, key);
+    if (buckets) warp_bucket_cells(a, p_out, emit, key, r);
+    else warp_count_cells(a.count[p_out], emit, key);
 }
 
 constexpr uint32_t kGridPolls = 1u << 22;  // bound of every grid-barrier wait (polls of ~0.1 us)
 
 // Grid-wide barrier of a cooperative launch (every block resident): the blocks' thread 0 count in on
-// a global counter; the last to arrive resets it and advances the generation the others poll.  Bounded:
-// false after kGridPolls polls (the caller reports KNS_ERR_TIMEOUT and leaves).  Block-uniform result.
-__device__ __forceinline__ bool grid_sync(WaveCtrl *ctrl, unsigned &gen, int *s_flag, uint32_t polls = kGridPolls) {
+// a global counter; the last to arrive resets it, runs `last` and advances the generation the others poll.
+// Bounded: false after kGridPolls polls (the caller reports KNS_ERR_TIMEOUT and leaves).  Block-uniform result.
+struct NothingLast {
+    __device__ void operator()() const {}
+};
+template <class F = NothingLast>
+__device__ __forceinline__ bool grid_sync(WaveCtrl *ctrl, unsigned &gen, int *s_flag, uint32_t polls = kGridPolls,
+                                          F last = F{}) {
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
@@ -280,6 +305,7 @@ __device__ __forceinline__ bool grid_sync(WaveCtrl *ctrl, unsigned &gen, int *s_
         __threadfence();
         if (atomicAdd(&ctrl->bar_count, 1u) == gridDim.x - 1) {
             atomicExch(&ctrl->bar_count, 0u);
+            last();
             __threadfence();
             atomicExch(&ctrl->bar_gen, target);
         } else {
