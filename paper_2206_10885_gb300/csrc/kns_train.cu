@@ -27,6 +27,11 @@ using train::fd_normal;
 using train::grid_for;
 using train::load3;
 
+// threads per block of the kernels that walk a ray's samples in turn: one warp, so that the 1,024 rays of a small
+// batch spread over 32 SMs
+constexpr int RAYS = 32;
+unsigned ray_blocks(int64_t rays) { return (unsigned)((rays + RAYS - 1) / RAYS); }
+
 // ------------------------------------------------------------------ activations
 __device__ __forceinline__ float sigm(float s) { return 1.f / (1.f + expf(-s)); }
 // log sigmoid(x), stable for any x
@@ -203,7 +208,7 @@ __global__ void __launch_bounds__(256) k_scatter(TrainArgs a, int64_t n) {
 }
 
 // ------------------------------------------------------------------ importance sampling
-__global__ void __launch_bounds__(128) k_importance(TrainArgs a) {
+__global__ void __launch_bounds__(RAYS) k_importance(TrainArgs a) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= a.B) return;
     float o[3], w[3], tn, tf;
@@ -221,10 +226,11 @@ __global__ void __launch_bounds__(128) k_importance(TrainArgs a) {
     for (int i = 0; i < Ns; ++i) tc[i] = strat_t(tn, tf, i, __ldg(a.u_s + r * Ns + i), Ns);
     // coarse NeuS weights on the Ns - 1 intervals (+1e-5 floor), cumulated
     const float *dc = a.d_coarse + r * Ns;
-    float T = 1.f, tot = 0.f, ls = log_sigm(a.s_up * dc[0]);
+    float T = 1.f, tot = 0.f, ls = log_sigm(a.s_up * __ldg(dc));
     cdf[0] = 0.f;
+#pragma unroll 4
     for (int i = 0; i + 1 < Ns; ++i) {
-        const float ls1 = log_sigm(a.s_up * dc[i + 1]);
+        const float ls1 = log_sigm(a.s_up * __ldg(dc + i + 1));
         const float alpha = fmaxf(1.f - expf(ls1 - ls), 0.f);
         tot += T * alpha + 1e-5f;
         T *= 1.f - alpha;
@@ -277,21 +283,24 @@ __device__ __forceinline__ void block_add(double v, double *dst) {
     }
 }
 
-__global__ void __launch_bounds__(128) k_composite_fwd(TrainArgs a, float *rgb_out) {
+__global__ void __launch_bounds__(RAYS) k_composite_fwd(TrainArgs a, float *rgb_out) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double l1 = 0.0;
     if (r < a.B) {
         float C[3] = {0.f, 0.f, 0.f};
         if (a.valid[r]) {
             const int64_t q0 = r * a.S;
-            float Tr = 1.f, ls = log_sigm(a.s * a.d_c[q0]);
+            const float *dc = a.d_c + q0, *rgb = a.rgb_c + 3 * q0;
+            float Tr = 1.f, ls = log_sigm(a.s * __ldg(dc));
+            // (the read-only loads of several samples go out together: a small batch has few warps to wait in turn)
+#pragma unroll 4
             for (int i = 0; i + 1 < a.S; ++i) {
-                const float ls1 = log_sigm(a.s * a.d_c[q0 + i + 1]);
+                const float ls1 = log_sigm(a.s * __ldg(dc + i + 1));
                 const float alpha = fmaxf(1.f - expf(ls1 - ls), 0.f);
                 const float wgt = Tr * alpha;
-                C[0] = fmaf(wgt, a.rgb_c[3 * (q0 + i)], C[0]);
-                C[1] = fmaf(wgt, a.rgb_c[3 * (q0 + i) + 1], C[1]);
-                C[2] = fmaf(wgt, a.rgb_c[3 * (q0 + i) + 2], C[2]);
+                C[0] = fmaf(wgt, __ldg(rgb + 3 * i), C[0]);
+                C[1] = fmaf(wgt, __ldg(rgb + 3 * i + 1), C[1]);
+                C[2] = fmaf(wgt, __ldg(rgb + 3 * i + 2), C[2]);
                 Tr *= 1.f - alpha;
                 ls = ls1;
             }
@@ -326,7 +335,7 @@ __global__ void k_finalize(TrainArgs a) {
 }
 
 // upstream of the sample centres' d and colour from dL/dC = sign(C - I) dloss / B
-__global__ void __launch_bounds__(128) k_composite_bwd(TrainArgs a) {
+__global__ void __launch_bounds__(RAYS) k_composite_bwd(TrainArgs a) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= a.B || !a.valid[r]) return;
     const float dl = a.dloss ? *a.dloss : 1.f;
@@ -338,11 +347,13 @@ __global__ void __launch_bounds__(128) k_composite_bwd(TrainArgs a) {
     }
     const int64_t q0 = r * a.S;
     const int S = a.S;
+    const float *dc = a.d_c + q0, *rgb = a.rgb_c + 3 * q0;
     float Tl[MAXS];
     {
-        float Tr = 1.f, ls = log_sigm(a.s * a.d_c[q0]);
+        float Tr = 1.f, ls = log_sigm(a.s * __ldg(dc));
+#pragma unroll 4
         for (int i = 0; i + 1 < S; ++i) {
-            const float ls1 = log_sigm(a.s * a.d_c[q0 + i + 1]);
+            const float ls1 = log_sigm(a.s * __ldg(dc + i + 1));
             Tl[i] = Tr;
             Tr *= 1.f - fmaxf(1.f - expf(ls1 - ls), 0.f);
             ls = ls1;
@@ -352,13 +363,14 @@ __global__ void __launch_bounds__(128) k_composite_bwd(TrainArgs a) {
     float Ch[3] = {0.f, 0.f, 0.f};
     float dd_next = 0.f;
     a.g_rgb[3 * (q0 + S - 1)] = a.g_rgb[3 * (q0 + S - 1) + 1] = a.g_rgb[3 * (q0 + S - 1) + 2] = 0.f;
-    float d1 = a.d_c[q0 + S - 1];
+    float d1 = __ldg(dc + S - 1);
+#pragma unroll 4
     for (int i = S - 2; i >= 0; --i) {
-        const float d0 = a.d_c[q0 + i];
+        const float d0 = __ldg(dc + i);
         const float ls0 = log_sigm(a.s * d0), ls1 = log_sigm(a.s * d1);
         const float rho = expf(ls1 - ls0);
         const float alpha = fmaxf(1.f - rho, 0.f);
-        const float c0 = a.rgb_c[3 * (q0 + i)], c1 = a.rgb_c[3 * (q0 + i) + 1], c2 = a.rgb_c[3 * (q0 + i) + 2];
+        const float c0 = __ldg(rgb + 3 * i), c1 = __ldg(rgb + 3 * i + 1), c2 = __ldg(rgb + 3 * i + 2);
         const float dalpha = Tl[i] * (gC[0] * (c0 - Ch[0]) + gC[1] * (c1 - Ch[1]) + gC[2] * (c2 - Ch[2]));
         float dd0 = 0.f;
         if (1.f - rho > 0.f) {
@@ -413,7 +425,7 @@ cudaError_t train_sort(const TrainArgs &a, int which, int64_t n_rec, int sm_coun
 
 cudaError_t train_importance(const TrainArgs &a, cudaStream_t s) {
     if (a.B == 0) return cudaSuccess;
-    k_importance<<<(unsigned)((a.B + 127) / 128), 128, 0, s>>>(a);
+    k_importance<<<ray_blocks(a.B), RAYS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -426,7 +438,7 @@ cudaError_t train_valid(const TrainArgs &a, cudaStream_t s) {
 cudaError_t train_loss_forward(const TrainArgs &a, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(a.acc, 0, 2 * sizeof(double), s);
     if (e != cudaSuccess) return e;
-    if (a.B > 0) k_composite_fwd<<<(unsigned)((a.B + 127) / 128), 128, 0, s>>>(a, nullptr);
+    if (a.B > 0) k_composite_fwd<<<ray_blocks(a.B), RAYS, 0, s>>>(a, nullptr);
     if (a.M > 0) k_eik_fwd<<<(unsigned)((a.M + 127) / 128), 128, 0, s>>>(a);
     k_finalize<<<1, 1, 0, s>>>(a);
     return cudaGetLastError();
@@ -438,7 +450,7 @@ cudaError_t train_rgb_out(const TrainArgs &a, float *rgb, cudaStream_t s) {
 }
 
 cudaError_t train_upstream(const TrainArgs &a, cudaStream_t s) {
-    if (a.B > 0) k_composite_bwd<<<(unsigned)((a.B + 127) / 128), 128, 0, s>>>(a);
+    if (a.B > 0) k_composite_bwd<<<ray_blocks(a.B), RAYS, 0, s>>>(a);
     if (a.M > 0) k_eik_bwd<<<(unsigned)((a.M + 127) / 128), 128, 0, s>>>(a);
     return cudaGetLastError();
 }

@@ -12,8 +12,10 @@
 // What bounds them is the FP32 pipe and the loads that feed it.  Block tiles of 128 records (a barrier per layer;
 // for each layer's weight gradient only the 72 threads that held its entries at work) took, per step of 65,536 rays
 // x 96 samples and 16,384 eikonal points on a GB300: difference points forward 7.1 ms, centres forward 2.5,
-// centres backward 10.6, difference points backward 28.6 ms; now 6.3, 2.2, 7.2 and 24.7 ms (the step 51.3 -> 42.4
-// ms; 1,024 rays 3.0 -> 2.5 ms).
+// centres backward 10.6, difference points backward 28.6 ms; now 6.3, 2.2, 7.1 and 18.8 ms (the step 51.2 -> 36.6
+// ms; 1,024 rays 3.0 -> 2.2 ms).  The forward kernel keeps the FP32 pipe 58 % busy; the backward ones have eight
+// warps of 255 registers per SM and wait on shared loads and instruction fetch: unrolling the weight-gradient
+// loop twice costs 4.7 ms, five warps of 168 registers the same, loads a half step ahead 2.9 ms.
 //
 // Kernels: d at records (coarse samples and difference points); sample centres forward (d, z,
 // colour); sample centres backward (colour and SDF, writes the difference points' upstream);
@@ -112,9 +114,9 @@ __device__ __forceinline__ void encode_record(float *E, int lane, float x, float
 }
 
 // ------------------------------------------------------------------ forward: d at records
-constexpr int FW = 8;  // warps per block
+constexpr int FW = 8, FB = 3;  // warps per block, blocks per SM
 template <int H>
-__global__ void __launch_bounds__(32 * FW, 2) k_warp_eval_d(TrainArgs a, int k0, int k1, float *out) {
+__global__ void __launch_bounds__(32 * FW, FB) k_warp_eval_d(TrainArgs a, int k0, int k1, float *out) {
     using S = WW<H>;
     extern __shared__ float4 smem4[];
     float *sw = reinterpret_cast<float *>(smem4);
@@ -140,7 +142,7 @@ __global__ void __launch_bounds__(32 * FW, 2) k_warp_eval_d(TrainArgs a, int k0,
             __syncwarp();  // every lane has read the input before it is overwritten
             m.store(rows, WRS, act);
             __syncwarp();
-#pragma unroll
+#pragma unroll 1
             for (int l = 1; l < H; ++l) {
                 m.bias_shared(sw + S::b(l));
                 m.template mm_shared<32>(sw + S::T(l), WTS, rows, WRS);
@@ -164,7 +166,7 @@ __global__ void __launch_bounds__(32 * FW, 2) k_warp_eval_d(TrainArgs a, int k0,
 // of the whole chunk stay in registers -- lane (og, ig) = (lane / 8, lane % 8) owns outputs og + 4 i and inputs
 // ig + 8 j of every layer, 12 loads of 16 bytes for 128 FMAs -- and are summed over the block's warps in shared
 // memory and added to the global gradient once per chunk.
-constexpr int BW = 5;  // warps per block, two blocks per SM
+constexpr int BW = 4;  // warps per block, two blocks per SM: 255 registers, 101 of them gradient sums
 template <int H>
 struct WRows {
     __host__ __device__ static constexpr int A(int l) { return 32 * l; }  // A(0): the encoding
@@ -172,26 +174,26 @@ struct WRows {
 };
 
 // acc[i][j] += sum over the tile's records of D[og + 4 i] A[ig + 8 j]
+__device__ __forceinline__ void fma44(const float4 &dv, const float4 (&xv)[4], float (&acc)[4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        float s = acc[j];
+        s = fmaf(dv.x, xv[j].x, s);
+        s = fmaf(dv.y, xv[j].y, s);
+        s = fmaf(dv.z, xv[j].z, s);
+        s = fmaf(dv.w, xv[j].w, s);
+        acc[j] = s;
+    }
+}
 __device__ __forceinline__ void grad_tile32(const float *D, const float *A, float (&acc)[8][4], int lane) {
     const float *d = D + (lane >> 3) * WRS, *x = A + (lane & 7) * WRS;
-#pragma unroll 2
+#pragma unroll 1
     for (int r = 0; r < WT; r += 4) {
         float4 xv[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) xv[j] = *reinterpret_cast<const float4 *>(x + 8 * j * WRS + r);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float4 dv = *reinterpret_cast<const float4 *>(d + 4 * i * WRS + r);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                float s = acc[i][j];
-                s = fmaf(dv.x, xv[j].x, s);
-                s = fmaf(dv.y, xv[j].y, s);
-                s = fmaf(dv.z, xv[j].z, s);
-                s = fmaf(dv.w, xv[j].w, s);
-                acc[i][j] = s;
-            }
-        }
+        for (int i = 0; i < 8; ++i) fma44(*reinterpret_cast<const float4 *>(d + 4 * i * WRS + r), xv, acc[i]);
     }
 }
 // sum over the tile's records of row `lane` of X times g (NULL: 1)
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(32 * BW, 2) k_warp_fd_backward(TrainArgs a) {
             m.template mm_shared<28>(sw + S::T(0), WTS, rows, WRS);
             m.store(rows + R::A(1) * WRS, WRS, act);
             __syncwarp();
-#pragma unroll
+#pragma unroll 1
             for (int l = 1; l < H; ++l) {
                 m.bias_shared(sw + S::b(l));
                 m.template mm_shared<32>(sw + S::T(l), WTS, rows + R::A(l) * WRS, WRS);
@@ -374,10 +376,11 @@ struct CR {
 };
 
 // A tile forward: lane j and lane j + 16 share record j (q < 0: padding).  Leaves the activations, d and z, the
-// colour inputs and the colour hidden layer in the rows; returns the colour logits in lanes 0 .. 15.
+// colour inputs and the colour hidden layer in the rows; returns the colour logits and the difference gradient's
+// length in lanes 0 .. 15.
 template <int H, bool KEEP>
 __device__ __forceinline__ void centre_tile(const TrainArgs &a, const float *sw, float *rows, int lane, float4 r,
-                                            long long q, float (&lg)[3]) {
+                                            long long q, float (&lg)[3], float &gn) {
     using W = WW<H>;
     using S = WC<H>;
     using R = CR<H, KEEP>;
@@ -389,7 +392,7 @@ __device__ __forceinline__ void centre_tile(const TrainArgs &a, const float *sw,
             for (int c = 0; c < 3; ++c) rows[c * CRS + j] = p[c];
             if (!KEEP) rows[27 * CRS + j] = 0.f;
             float n[3] = {0.f, 0.f, 0.f}, g[3];
-            if (q >= 0) fd_normal(a, q, g, n);
+            if (q >= 0) gn = fd_normal(a, q, g, n);
 #pragma unroll
             for (int c = 0; c < 3; ++c) rows[(R::U + 15 + c) * CRS + j] = n[c];
         } else {
@@ -493,8 +496,8 @@ __global__ void __launch_bounds__(32 * CFW, 2) k_warp_centre_fwd(TrainArgs a) {
                 r = a.sorted[i];
                 q = (long long)__float_as_int(r.w) - nfd;
             }
-            float lg[3];
-            centre_tile<H, false>(a, sw, rows, lane, r, q, lg);
+            float lg[3], gn;
+            centre_tile<H, false>(a, sw, rows, lane, r, q, lg, gn);
             if (lane < 16 && q >= 0) {
                 a.d_c[q] = rows[R::Ud * CRS + lane];
                 a.rgb_c[3 * q] = sigm(lg[0]);
@@ -516,18 +519,7 @@ __device__ __forceinline__ void grad_tile16(const float *D, const float *A, floa
 #pragma unroll
         for (int j = 0; j < 4; ++j) xv[j] = *reinterpret_cast<const float4 *>(x + 8 * j * CRS + r);
 #pragma unroll
-        for (int i = 0; i < NI; ++i) {
-            const float4 dv = *reinterpret_cast<const float4 *>(d + 4 * i * CRS + r);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                float s = acc[i][j];
-                s = fmaf(dv.x, xv[j].x, s);
-                s = fmaf(dv.y, xv[j].y, s);
-                s = fmaf(dv.z, xv[j].z, s);
-                s = fmaf(dv.w, xv[j].w, s);
-                acc[i][j] = s;
-            }
-        }
+        for (int i = 0; i < NI; ++i) fma44(*reinterpret_cast<const float4 *>(d + 4 * i * CRS + r), xv, acc[i]);
     }
 }
 // sum over the tile's records of x times y (y NULL: 1), rows of CT records
@@ -594,17 +586,22 @@ __global__ void __launch_bounds__(32 * CBW, 1) k_warp_centre_backward(TrainArgs 
                 r = a.sorted[i];
                 q = (long long)__float_as_int(r.w) - nfd;
             }
-            float lg[3];
-            centre_tile<H, true>(a, sw, rows, lane, r, q, lg);
+            float lg[3], gn = 0.f, up[4] = {0.f, 0.f, 0.f, 0.f};
+            if (lane < 16 && q >= 0) {  // the upstreams, on their way while the tile runs forward
+#pragma unroll
+                for (int c = 0; c < 3; ++c) up[c] = a.g_rgb[3 * q + c];
+                up[3] = a.g_dc[q];
+            }
+            centre_tile<H, true>(a, sw, rows, lane, r, q, lg, gn);
             if (lane < 16) {  // logits -> colour delta; the upstream of d
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     const float rgb = sigm(lg[c]);
-                    const float dc = q >= 0 ? a.g_rgb[3 * q + c] * rgb * (1.f - rgb) : 0.f;
+                    const float dc = up[c] * rgb * (1.f - rgb);
                     rows[(R::Dc + c) * CRS + lane] = dc;
                     dbc1[c] += dc;
                 }
-                rows[R::Dout * CRS + lane] = q >= 0 ? a.g_dc[q] : 0.f;
+                rows[R::Dout * CRS + lane] = up[3];
             }
             __syncwarp();
 #pragma unroll
@@ -632,8 +629,8 @@ __global__ void __launch_bounds__(32 * CBW, 1) k_warp_centre_backward(TrainArgs 
             m.store(rows + R::Hc * CRS, CRS, [](float v, int, int) { return v; });
             __syncwarp();
             if (lane < 16 && q >= 0) {  // the normal's delta to the difference records
-                float g[3], n[3];
-                const float gn = fd_normal(a, q, g, n);
+                const float n[3] = {rows[(R::U + 15) * CRS + lane], rows[(R::U + 16) * CRS + lane],
+                                    rows[(R::U + 17) * CRS + lane]};
                 const float gx = rows[(R::Hc + 15) * CRS + lane], gy = rows[(R::Hc + 16) * CRS + lane],
                             gz = rows[(R::Hc + 17) * CRS + lane];
                 const float nd = n[0] * gx + n[1] * gy + n[2] * gz;
@@ -724,7 +721,7 @@ cudaError_t eval_d_h(const TrainArgs &a, int k0, int k1, float *out, int64_t chu
     const size_t sm = (WW<H>::FEND + FW * 32 * WRS) * sizeof(float);
     cudaError_t e = set_smem(k_warp_eval_d<H>, sm);
     if (e != cudaSuccess) return e;
-    k_warp_eval_d<H><<<grid_for(sm_count, 2, chunks), 32 * FW, sm, s>>>(a, k0, k1, out);
+    k_warp_eval_d<H><<<grid_for(sm_count, FB, chunks), 32 * FW, sm, s>>>(a, k0, k1, out);
     return cudaGetLastError();
 }
 
