@@ -134,8 +134,8 @@ typedef struct kns_render_opts {
     int32_t static_tiles;  /* 1: each block takes a contiguous run of tiles; 2: tiles handed out dynamically */
     int32_t timing;        /* 1: time each kernel class with CUDA events for kns_get_render_stats (adds host work) */
     int32_t block_tiles;   /* FP32 evaluation (KNS_FP32 renders): 1 = 128-sample tiles per
-                              256-thread block (block GEMMs); 3 = 256-sample tiles per 256 threads; 4 = 128-sample
-                              tiles per 128 threads; 2 = 16-sample tiles per warp (in-tile stepping, min_active);
+                              256-thread block (block GEMMs); 3 = 256-sample tiles per 256 threads; 4 = tiles of 128
+                              split between warps that step their own samples (32, or 16 at SDF width 64); 2 = 16-sample tiles per warp (in-tile stepping, min_active);
                               0 = default (4) */
     int32_t bf16_inner_steps; /* KNS_BF16: evaluations a tensor-core tile may make per round while its rays stay in
                                  its cell (1..1024; default 4 at SDF width 32, 2 at width 64) */

@@ -8,6 +8,7 @@
 // s = sample); lane (sg, ng) = (lane / 8, lane % 8) accumulates samples 4sg..4sg+3 against output
 // units ng*W/8 .. ng*W/8 + W/8 - 1, so each shared-memory float4 of activations and each float4 of
 // k-major weights feed 16 (W = 32) or 32 (W = 64) FMAs.
+#include "kns_warp.cuh"
 #include "kns_wave.cuh"
 
 namespace kns {
@@ -464,6 +465,213 @@ __global__ void __launch_bounds__(NT, block_min_blocks<C, BT>()) wave_eval_block
     }
 }
 
+// ---------------------------------------------------------------- warp-private block tiles (FP32 default)
+// A tile of up to 128 samples of one cell as above, its weights staged once for the block, but every warp takes its
+// own samples -- 32 at width 32, 16 at width 64 -- through all layers on rows of its own (kns_warp.cuh; a layer
+// overwrites its input), tests and steps them, and evaluates those that stay in the cell again, up to inner_steps
+// times while enough of them do, without a barrier: the block's warps meet only where the next tile's weights
+// replace this one's.  d is the same sum, so results do not depend on the tile shape.
+// Bound by the FMA pipe and by the rounds' serial chain: the shared tiles lost their time at a barrier per layer and
+// per pass, which every warp reached when the slowest did.  Two 1080p views of the 16^3 width-32 grid 6.64 -> 6.18 ms,
+// two of the 32^3 width-64 grid 9.67 -> 9.10 ms, four 640 x 480 views 2.16 -> 2.05 ms.  Loading the next tile's weights
+// into a second buffer gained nothing, five blocks an SM (a spill) and 16 samples a warp at width 32 were slower.
+template <class C>
+struct EB {
+    static constexpr int P = C::W == 32 ? 32 : 16, NW = 128 / P, NT = 32 * NW, BLOCKS = C::W == 32 ? 4 : 2;
+    static constexpr int ROWS = C::INP > C::W ? C::INP : C::W, RS = row_stride(P);
+    static constexpr int SMEM = (C::TSIZE + NW * ROWS * RS) * 4;
+};
+
+template <class C, bool STACK>
+__global__ void __launch_bounds__(EB<C>::NT, EB<C>::BLOCKS) wave_eval_warps_kernel(GridView g, WaveArgs a, int cur) {
+    using B = EB<C>;
+    constexpr int P = B::P, RS = B::RS, NH = 32 / P, W = C::W;
+    extern __shared__ __align__(128) float dyn[];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ int s_tile[2][4];  // cell, start, len, fresh; alternating
+    __shared__ int s_fail;
+    if (a.ctrl->tail) return;  // finished one warp per ray by wave_tail_warp_kernel
+    const int n_tiles = a.ctrl->n_tiles_fine;
+    if (n_tiles <= 0) return;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nxt = cur ^ 1;
+    float *wsm = dyn, *A = dyn + C::TSIZE + warp * B::ROWS * RS;
+    if (tid == 0) {
+        mbar_init(&bar, 1);
+        s_fail = 0;
+    }
+    const int per = (n_tiles + gridDim.x - 1) / gridDim.x;
+    int next_static = blockIdx.x * per;
+    const int end_static = min(n_tiles, next_static + per);
+    const int keep = max(1, a.min_active * P / 128);  // samples a warp goes on for
+    const bool cycles = a.t_hist != nullptr;
+    uint32_t phase = 0;
+    // thread 0 keeps two tiles in flight: the next one's descriptor (loaded) and the index after it (claimed)
+    int4 nd = make_int4(-1, 0, 0, 0);
+    int nt = n_tiles, cached = -1;
+    unsigned n_eval = 0;
+    if (tid == 0) {
+        const int t0 = claim_tile(a, n_tiles, next_static, end_static);
+        if (t0 < n_tiles) nd = a.tiles[t0];
+        nt = claim_tile(a, n_tiles, next_static, end_static);
+    }
+    for (int par = 0;; par ^= 1) {
+        if (tid == 0) {
+            s_tile[par][0] = nd.x;
+            s_tile[par][1] = nd.y;
+            s_tile[par][2] = nd.z;
+            s_tile[par][3] = nd.x != cached;
+        }
+        __syncthreads();  // and every warp is done with the previous tile's weights
+        const int c = s_tile[par][0], start = s_tile[par][1], len = s_tile[par][2];
+        bool wait = s_tile[par][3] != 0;
+        if (c < 0 || s_fail) break;
+        cached = c;
+        if (tid == 0) {
+            if (wait) bulk_load(wsm, a.wt + (int64_t)c * a.wt_stride, C::TSIZE * sizeof(float), &bar);
+            nd = nt < n_tiles ? a.tiles[nt] : make_int4(-1, 0, 0, 0);
+            if (nt < n_tiles) nt = claim_tile(a, n_tiles, next_static, end_static);
+        }
+        const int first = warp * P + lane;
+        bool active = lane < P && first < len;
+        int r = 0, steps = 0;
+        float t = 0.f, t0 = 0.f, tf = 0.f;
+        float4 hist = no_history();
+        Ray ray{};
+        if (active) {
+            r = a.sorted[start + first];
+            t = a.t_ray[r];
+            if (cycles) hist = a.t_hist[r];
+            steps = a.steps_ray[r];
+            int cam;
+            ray = ray_of(a, r, cam);
+            clip_box(g, ray, t0, tf);
+        }
+        for (int it = 0; __any_sync(FULL, active); ++it) {
+            {  // Eq. 1, NH lanes per sample sharing the frequencies
+                const int j = lane % P, h = lane / P;
+                float p[3] = {fmaf(t, ray.wx, ray.ox), fmaf(t, ray.wy, ray.oy), fmaf(t, ray.wz, ray.oz)};
+                if (NH > 1)
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) p[q] = __shfl_sync(FULL, p[q], j);
+                if (h == 0) {
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) A[q * RS + j] = p[q];
+#pragma unroll
+                    for (int k = C::IN; k < C::INP; ++k) A[k * RS + j] = 0.f;
+                }
+#pragma unroll
+                for (int kk = 0; kk < C::L / NH; ++kk) {
+                    const int k = kk * NH + h;
+                    const float f = (float)(1 << k);
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        float sn, cs;
+                        sincospif(f * p[q], &sn, &cs);
+                        A[(3 + 6 * k + q) * RS + j] = sn;
+                        A[(6 + 6 * k + q) * RS + j] = cs;
+                    }
+                }
+            }
+            if (wait) {
+                wait = false;
+                if (!__all_sync(FULL, mbar_wait(&bar, phase, 1u << 26))) {  // the weights never landed: report
+                    if (lane == 0) {
+                        atomicCAS(a.status, 0, (int)6 /* KNS_ERR_TIMEOUT */);
+                        s_fail = 1;
+                    }
+                    break;
+                }
+                phase ^= 1u;
+            }
+            __syncwarp();
+            TileMap<W, P> m(lane);
+            auto act = [&](float v, int, int) { return softplus_f32(v, g.beta, g.inv_beta); };
+            m.bias_shared(wsm + C::tb0);
+            m.template mm_shared<C::INP>(wsm + C::tW0, W, A, RS);
+            __syncwarp();  // every lane has read the input before it is overwritten
+            m.store(A, RS, act);
+            __syncwarp();
+#pragma unroll 1
+            for (int l = 1; l < C::H; ++l) {
+                m.bias_shared(wsm + C::tbl(l));
+                m.template mm_shared<W>(wsm + C::tWl(l), W, A, RS);
+                __syncwarp();
+                m.store(A, RS, act);
+                __syncwarp();
+            }
+            // the d row: bias first, then one sequential FMA chain over k
+            float d = wsm[C::tbL];
+            {
+                const float *h = A + (lane % P);
+#pragma unroll 8
+                for (int k = 0; k < W; ++k) d = fmaf(wsm[C::tdL + k], h[k * RS], d);
+            }
+            __syncwarp();
+            // outcome: 0 none (inactive), 1 hit, 2 miss (written), 3 pending, 4 emit to ncell
+            int outcome = 0, ncell = -1;
+            const float t_eval = t;
+            if (active) {
+                ++n_eval;
+                ++steps;
+                if (fabsf(d) < a.eps) {
+                    outcome = 1;
+                } else {
+                    t += d;
+                    if (t > tf || t < t0 || steps >= a.max_steps) {
+                        outcome = 2;
+                        write_miss(a, r, steps);
+                    } else {
+                        // an occupied voxel gives the next cell at once; a ray that stepped into empty space goes on
+                        // the round's pending list for wave_advance_kernel, so that no lane holds the warp in a
+                        // long voxel walk
+                        if constexpr (STACK) ncell = advance_fast(sub_grid(g, c / g.ncl), ray, t);
+                        else ncell = advance_fast(g, ray, t);
+                        if (ncell == -2) {
+                            outcome = 3;
+                        } else if (cycles && cycle_step(hist, t_eval, t)) {
+                            outcome = 2;
+                            write_miss(a, r, a.max_steps);
+                        } else {
+                            outcome = 4;
+                        }
+                    }
+                }
+            }
+            // samples that stay in this cell are evaluated again while enough of the warp's do
+            const bool cand = outcome == 4 && ncell == c && it + 1 < a.inner_steps;
+            const unsigned stays = __ballot_sync(FULL, cand);
+            const bool stay = cand && __popc(stays) >= keep;
+            const bool hit = outcome == 1, emit = outcome == 4 && !stay, pend = outcome == 3;
+            if (hit) a.cell_ray[r] = c;
+            if (hit || emit || pend) {
+                a.t_ray[r] = t;
+                a.steps_ray[r] = steps;
+                if (cycles && !hit) a.t_hist[r] = hist;
+            }
+            const int hp = warp_append(&a.ctrl->n_hits, hit);
+            if (hit) a.hits[hp] = r;
+            const int qp = warp_append(&a.ctrl->n_live[nxt], emit);
+            if (emit) {
+                a.q[nxt][qp] = r;
+                a.qcell[nxt][qp] = ncell;
+            }
+            warp_count_cells(a.count[nxt], emit, ncell);
+            const int pp = warp_append(&a.ctrl->n_pend[cur], pend);
+            if (pend) {
+                a.pend_r[cur][pp] = r;
+                a.pend_t[cur][pp] = t_eval;
+            }
+            active = stay;
+        }
+        if (wait) {  // a warp without samples follows the weights' phase
+            if (!mbar_wait(&bar, phase, 1u << 26)) s_fail = 1;
+            phase ^= 1u;
+        }
+    }
+    const unsigned long long n = warp_sum_u64(n_eval);
+    if (lane == 0 && n) atomicAdd(&a.ctrl->samples_f32, n);
+}
+
 // Tail: a warp runs one ray to its end.  The warp keeps the k-major trace weights of its ray's
 // current cell in a shared-memory slot of its own (one bulk copy per change of cell: the rays left
 // for the tail are mostly grazing rays that take many small steps inside one cell) and evaluates a
@@ -872,14 +1080,27 @@ cudaError_t launch_block_eval(const GridView &g, const WaveArgs &a, int cur, int
 }
 
 template <class C>
+cudaError_t launch_warps_eval(const GridView &g, const WaveArgs &a, int cur, int sm_count, cudaStream_t s) {
+    using B = EB<C>;
+    static std::atomic<int> single{0}, stack{0};
+    int nb = 0;
+    cudaError_t e = g.sub_boxes ? resident_blocks(wave_eval_warps_kernel<C, true>, B::NT, B::SMEM, stack, nb)
+                                : resident_blocks(wave_eval_warps_kernel<C, false>, B::NT, B::SMEM, single, nb);
+    if (e != cudaSuccess) return e;
+    if (g.sub_boxes) wave_eval_warps_kernel<C, true><<<sm_count * nb, B::NT, B::SMEM, s>>>(g, a, cur);
+    else wave_eval_warps_kernel<C, false><<<sm_count * nb, B::NT, B::SMEM, s>>>(g, a, cur);
+    return cudaGetLastError();
+}
+
+template <class C>
 cudaError_t launch_wave_eval_cfg(const GridView &g, const WaveArgs &a, int cur, int blocks, int block_tiles,
                                  int sm_count, cudaStream_t s) {
     cudaError_t e;
     if (block_tiles) {
-        // the sort's tile size decides the kernel: 256- or 128-sample block tiles, the latter with 256
-        // threads (two per sample in the encoding) or 128 (block_tiles == 4: one thread per sample)
+        // the sort's tile size decides the kernel: 256- or 128-sample block tiles of 256 threads, or (block_tiles == 4)
+        // 128-sample tiles split between the warps
         e = a.btile == 256 ? launch_block_eval<C, 256, 256>(g, a, cur, sm_count, s)
-            : block_tiles == 4 ? launch_block_eval<C, 128, 128>(g, a, cur, sm_count, s)
+            : block_tiles == 4 ? launch_warps_eval<C>(g, a, cur, sm_count, s)
                                : launch_block_eval<C, 128, 256>(g, a, cur, sm_count, s);
         if (e != cudaSuccess) return e;
     } else {

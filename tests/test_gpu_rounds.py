@@ -48,3 +48,26 @@ def test_step_budget_ends_the_rounds(scene):
         ctx.sync()
         for k in a:
             assert torch.equal(a[k], b[k]), (steps, k)
+
+
+@pytest.mark.parametrize("width", [32, 64])
+@pytest.mark.parametrize("W,H", [(1, 1), (17, 1), (33, 4), (129, 3), (160, 96)])
+def test_warp_private_tiles(width, W, H):
+    """The default evaluator against the one whose blocks share their tiles: every sample is the same sum, so the
+    images are equal bit for bit, whatever the tile's remainder and however long a warp stays in a cell."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2206_10885_gb300 as kns
+    with kns.Context(0) as ctx:
+        for res in (0, 64):
+            desc = S.GridDesc(N=4, sdf_width=width, col_width=width, pe_pos_L=4 if width == 32 else 6,
+                              pe_dir_L=2 if width == 32 else 4, occ_res=res)
+            grid = kns.Grid.load(ctx, desc, S.sal_sphere_grid(desc))
+            cams = S.orbit_cameras(1, W, H, seed=7)
+            ref = kns.render(ctx, grid, cams, W, H, 64, 1e-4, tuning=dict(tail_rays=-1, block_tiles=1))
+            for tune in (dict(), dict(inner_steps=1), dict(inner_steps=64, min_active=1), dict(min_active=128)):
+                out = kns.render(ctx, grid, cams, W, H, 64, 1e-4, tuning=dict(tail_rays=-1, block_tiles=4, **tune))
+                ctx.sync()
+                for k in ref:
+                    assert torch.equal(out[k], ref[k]), (res, tune, k)
+            grid.free()
