@@ -168,7 +168,7 @@ template <class C>
 __device__ bool tc_round(TcWorker &w, const GridView &g, const WaveArgs &a, int cur, int n_tiles, int gi, int nw,
                          bool from_buckets = false, bool to_buckets = false) {
     using T = TcLayout<C>;
-    const int tid = w.tid, nxt = cur ^ 1;
+    const int tid = w.tid;
     const uint32_t w_base = tc::saddr(w.wsm), ta = w.tmem + (uint32_t)T::W;  // A_hi's first column
     const uint32_t t_lane = w.tmem + ((uint32_t)(32 * w.warp) << 16);       // this warp's lanes
     const uint32_t ta_lane = ta + ((uint32_t)(32 * w.warp) << 16);
@@ -361,20 +361,7 @@ __device__ bool tc_round(TcWorker &w, const GridView &g, const WaveArgs &a, int 
                 }
                 if (cycles && emit) a.t_hist[r] = hist;
                 if (a.trap && (emit || pend)) a.trap[r] = trap;
-                const int hp = warp_append(&a.ctrl->n_hits, hit);
-                if (hit) a.hits[hp] = r;
-                const int qp = warp_append(&a.ctrl->n_live[nxt], emit);
-                if (emit) {
-                    a.q[nxt][qp] = r;
-                    a.qcell[nxt][qp] = ncell;
-                }
-                if (to_buckets) warp_bucket_cells(a, nxt, emit, ncell, r);
-                else warp_count_cells(a.count[nxt], emit, ncell);
-                const int pp = warp_append(&a.ctrl->n_pend[cur], pend);
-                if (pend) {
-                    a.pend_r[cur][pp] = r;
-                    a.pend_t[cur][pp] = t_eval;
-                }
+                warp_queue(a, cur, hit, emit, pend, r, ncell, t_eval, to_buckets);
                 active = stay;
             }
             if (!again) break;

@@ -242,6 +242,51 @@ __device__ __forceinline__ void warp_bucket_cells(const WaveArgs &a, int p, bool
     }
 }
 
+// The ends of one evaluation of a round of parity cur, for a whole warp: hits to the hit list, rays left in empty
+// voxels to the round's pending list, and rays with a next sample to the next round's queue, counts and (buckets)
+// cell buckets.  The atomics that hand out the places are issued together, by lanes 0 to 2 and the groups' first
+// lanes, so the warp waits for one round trip to L2 instead of one per list: eight 1080p views of a 32^3 width-32
+// grid 13.72 -> 13.56 ms, one 511 x 383 view 2.58 -> 2.54 ms.
+__device__ __forceinline__ void warp_queue(const WaveArgs &a, int cur, bool hit, bool emit, bool pend, int r, int ncell,
+                                           float t_eval, bool buckets) {
+    const int nxt = cur ^ 1, lane = threadIdx.x & 31;
+    const unsigned mh = __ballot_sync(FULL, hit), mq = __ballot_sync(FULL, emit), mp = __ballot_sync(FULL, pend);
+    if (!(mh | mq | mp)) return;
+    unsigned grp = 0;
+    if (emit) grp = __match_any_sync(mq, ncell);
+    int rank = 0, base = 0;
+    if (emit && lane == __ffs(grp) - 1) {
+        if (buckets) rank = atomicAdd(a.count[nxt] + ncell, __popc(grp));
+        else atomicAdd(a.count[nxt] + ncell, __popc(grp));
+    }
+    {
+        const unsigned m = lane == 0 ? mh : lane == 1 ? mq : mp;
+        int *const at = lane == 0 ? &a.ctrl->n_hits : lane == 1 ? &a.ctrl->n_live[nxt] : &a.ctrl->n_pend[cur];
+        if (lane < 3 && m) base = atomicAdd(at, __popc(m));
+    }
+    const unsigned lt = lanemask_lt();
+    const int hp = __shfl_sync(FULL, base, 0) + __popc(mh & lt), qp = __shfl_sync(FULL, base, 1) + __popc(mq & lt),
+              pp = __shfl_sync(FULL, base, 2) + __popc(mp & lt);
+    if (hit) a.hits[hp] = r;
+    if (pend) {
+        a.pend_r[cur][pp] = r;
+        a.pend_t[cur][pp] = t_eval;
+    }
+    if (emit) {
+        a.q[nxt][qp] = r;
+        a.qcell[nxt][qp] = ncell;
+        if (buckets) {
+            rank = __shfl_sync(grp, rank, __ffs(grp) - 1) + __popc(grp & lt);
+            if (rank < kBucket) {
+                a.bucket[nxt][ncell * kBucket + rank] = r;
+                if ((rank & 127) == 0) a.list[nxt][atomicAdd(&a.ctrl->n_list[nxt], 1)] = ncell | (rank >> 7) << 18;
+            } else {
+                a.ctrl->over[nxt] = 1;
+            }
+        }
+    }
+}
+
 // Entry i of the pending list of parity p_in (i < n; every lane of the warp calls it): the ray walks the
 // occupancy DDA from its position to its next occupied voxel (or leaves the grid: a miss), takes the
 // cycle test on the position reached, and joins the queue, counts and live counter of parity p_out.
