@@ -111,6 +111,7 @@ struct kns_grid {
     int ws_stride = 0;              // floats per cell
     uint32_t *d_occ = nullptr;
     uint32_t *d_occ_coarse = nullptr;  // 8^3-voxel block mask (res % 8 == 0)
+    uint8_t *d_dist = nullptr;         // distance field of the mask (NULL: not kept)
     size_t occ_words64 = 0;
     int occ_box[6] = {0, 0, 0, -1, -1, -1};  // index box of the occupied voxels (lo xyz, hi xyz)
     int n_sub = 1;  // grids in the stack (kns_load_grid_stack): cells, layouts and masks back to back
@@ -340,6 +341,7 @@ void fill_view(kns_grid *g) {
     }
     v.occ = g->d_occ;
     v.occ_coarse = g->d_occ_coarse;
+    v.occ_dist = g->d_dist;
     v.cres = d.occ_res / 8;
     for (int a = 0; a < 3; ++a) {
         v.olo[a] = g->occ_box[a];
@@ -816,6 +818,15 @@ static kns_status load_grid_impl(kns_ctx *ctx, const kns_grid_desc *desc, const 
         if (e == cudaSuccess && occ_words)
             e = cudaMemcpy(g->d_occ, occ_words, g->occ_words64 * 8, cudaMemcpyHostToDevice);
         if (e == cudaSuccess && cw) e = cudaMalloc(&g->d_occ_coarse, cw * 4 * (size_t)n_sub);
+        // the distance field and a buffer to build it in; without the memory for them the walk uses the block mask
+        uint8_t *dist_tmp = nullptr;
+        const size_t nvox = (size_t)d.occ_res * d.occ_res * d.occ_res;
+        if (e == cudaSuccess && nvox * (size_t)n_sub <= kns::kOccDistBytes &&
+            (cudaMalloc(&g->d_dist, nvox * (size_t)n_sub) != cudaSuccess || cudaMalloc(&dist_tmp, nvox) != cudaSuccess)) {
+            cudaGetLastError();
+            cudaFree(g->d_dist);
+            g->d_dist = nullptr;
+        }
         fill_view(g);
         float diag = 0.f;
         for (int a = 0; a < 3; ++a) diag += g->view.ovox[a] * g->view.ovox[a];
@@ -828,10 +839,12 @@ static kns_status load_grid_impl(kns_ctx *ctx, const kns_grid_desc *desc, const 
                 kns::GridView v = g->view;
                 v.occ = nullptr;
                 v.occ_coarse = nullptr;
+                v.occ_dist = nullptr;
                 v.cell_base = (int)(k * ncl);  // grid k's cells
                 e = kns::launch_occupancy_f32(g->shape, v, diag, occ_k, 0);
                 if (e == cudaSuccess) e = cudaDeviceSynchronize();
             }
+            if (e == cudaSuccess && g->d_dist) e = kns::launch_occ_dist(occ_k, d.occ_res, dist_tmp, g->d_dist + nvox * k, 0);
             if (e == cudaSuccess && cw) {
                 e = kns::launch_coarse_occupancy(occ_k, d.occ_res, g->d_occ_coarse + cw * (size_t)k, 0);
                 if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -852,6 +865,8 @@ static kns_status load_grid_impl(kns_ctx *ctx, const kns_grid_desc *desc, const 
                 for (int a = 0; a < 6; ++a) boxes[6 * k + a] = init[a];
             }
         }
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        cudaFree(dist_tmp);
         for (int a = 0; a < 6; ++a) g->occ_box[a] = box[a];
         if (e == cudaSuccess && n_sub > 1) {  // each grid of a stack walks to its own box
             e = cudaMalloc(&g->d_boxes, boxes.size() * sizeof(int));
@@ -865,6 +880,7 @@ static kns_status load_grid_impl(kns_ctx *ctx, const kns_grid_desc *desc, const 
             cudaFree(g->d_ws);
             cudaFree(g->d_occ);
             cudaFree(g->d_occ_coarse);
+            cudaFree(g->d_dist);
             cudaFree(g->d_boxes);
             delete g;
             return cuda_err(ctx, e, "occupancy");
@@ -964,6 +980,7 @@ void kns_free_grid(kns_grid *g) {
         cudaFree(g->d_ws);
         cudaFree(g->d_occ);
         cudaFree(g->d_occ_coarse);
+        cudaFree(g->d_dist);
         cudaFree(g->d_boxes);
     }
     delete g;

@@ -245,6 +245,30 @@ __global__ void coarse_occupancy_kernel(const uint32_t *occ, int res, uint32_t *
     if ((threadIdx.x & 31) == 0 && b < nb) coarse[b >> 5] = ball;
 }
 
+// The distance field (GridView::occ_dist), one axis at a time: a Chebyshev distance is the minimum over the
+// neighbours along the last axis of the larger of that offset and the distance over the axes before it.
+__global__ void occ_dist_kernel(const uint32_t *occ, const uint8_t *in, uint8_t *out, int res, int axis) {
+    const int64_t n = (int64_t)res * res * res, v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= n) return;
+    const int64_t stride = axis == 0 ? 1 : axis == 1 ? res : (int64_t)res * res;
+    const int at = (int)((v / stride) % res);
+    int best = kOccDist;
+    for (int i = max(-kOccDist, -at); i <= min(kOccDist, res - 1 - at); ++i) {
+        const int64_t u = v + i * stride;
+        const int d = axis == 0 ? (((occ[u >> 5] >> (u & 31)) & 1u) ? 0 : kOccDist) : in[u];
+        best = min(best, max(abs(i), d));
+    }
+    out[v] = (uint8_t)best;
+}
+
+cudaError_t launch_occ_dist(const uint32_t *occ, int res, uint8_t *tmp, uint8_t *dist, cudaStream_t s) {
+    const unsigned blocks = (unsigned)(((int64_t)res * res * res + 255) / 256);
+    occ_dist_kernel<<<blocks, 256, 0, s>>>(occ, nullptr, dist, res, 0);
+    occ_dist_kernel<<<blocks, 256, 0, s>>>(occ, dist, tmp, res, 1);
+    occ_dist_kernel<<<blocks, 256, 0, s>>>(occ, tmp, dist, res, 2);
+    return cudaGetLastError();
+}
+
 // Index box of the occupied voxels: bounds[0..2] = the smallest x, y, z index of a set bit, bounds[3..5]
 // the largest (the caller initialises them to res and -1).  One thread per 32-bit word.
 __global__ void occ_bounds_kernel(const uint32_t *occ, int res, int *bounds) {
