@@ -128,7 +128,7 @@ typedef struct kns_render_opts {
     int32_t min_active;    /* a tile continues only while at least this many of its rays stay in its cell
                               (1..256; a warp tile holds 16; default 8 for warp tiles, 16 for block tiles) */
     int32_t tail_rays;     /* a round with at most this many rays is finished one warp per ray, in FP32 (>= 0;
-                              -1: never; default: KNS_FP32 131072 at SDF width 32, 32768 at width 64; KNS_BF16
+                              -1: never; default: KNS_FP32 98304 at SDF width 32, 32768 at width 64; KNS_BF16
                               32768 at width 32, 16384 at width 64) */
     int32_t blocks_per_sm; /* evaluation blocks (one warp each) launched per SM (1..64) */
     int32_t static_tiles;  /* 1: each block takes a contiguous run of tiles; 2: tiles handed out dynamically */

@@ -391,7 +391,11 @@ constexpr int kRenderInnerSteps = 4;
 constexpr int kRenderMinActive = 8;
 constexpr int kRenderBlockInnerSteps = 2;  // block tiles: a second evaluation of a tile in the round ...
 constexpr int kRenderBlockMinActive = 16;  // ... while at least 16 of its rays stay in its cell
-constexpr int kRenderTailRays = 131072;  // rounds this small finish one warp per ray (width 32)
+// FP32 rounds this small finish one warp per ray (width 32).  The tail takes a sample every ~205 cycles of an SM (its
+// shared memory: weights read once per sample, copied for half of them), a light round ~110 us; of 8,192 .. 196,608
+// rays (65,536 / 98,304 / 131,072): eight 800 x 800 views 6.28 / 6.30 / 6.32 ms, five views of a stack of two grids
+// 2.00 / 1.99 / 2.03 ms, 100,003 rays 0.68 / 0.67 / 0.67 ms.
+constexpr int kRenderTailRays = 98304;
 // Cells of all grids of a stack: the BF16 seam trap keeps a cell number in 19 bits.
 constexpr int64_t kMaxStackCells = 262144;
 // tensor-core tiles (BF16 renders): a second evaluation while at least 16 rays stay in the cell
@@ -401,7 +405,7 @@ constexpr int kRenderBf16MinActive = 16;
 // BF16 renders hand rounds of at most this many rays (live + pending) to the one-warp-per-ray FP32
 // tail: the best of 8K..512K on both 1080p workloads (a tensor-core round costs ~50 us however few its rays);
 // FP32 renders of width-64 grids too (their tail warps hold 41 KB of weights each: 5 per SM), the best of
-// 8K..512K on the 32^3 width-64 workload (131072 stays best at width 32)
+// 8K..512K on the 32^3 width-64 workload
 constexpr int kRenderBf16TailRays = 32768;
 constexpr int kRenderBf16TailRaysWide = 16384;  // BF16 renders of width-64 grids
 constexpr int kRenderBlocksPerSM = 16;
@@ -1040,7 +1044,7 @@ kns_status resolve_opts(kns_ctx *ctx, const kns_render_opts *opts, float eps, Re
     c.inner_steps = opts ? knob(opts->inner_steps, def_inner) : def_inner;
     c.min_active = opts ? knob(opts->min_active, def_min) : def_min;
     // the hand-over to the one-warp-per-ray tail and the BF16 tiles' in-tile evaluations, by width (the
-    // best of a sweep over 12,288 .. 131,072 rays and 1 .. 8 evaluations at 8 x 1920x1080): FP32 131,072 at
+    // best of a sweep over 12,288 .. 131,072 rays and 1 .. 8 evaluations at 8 x 1920x1080): FP32 98,304 at
     // width 32, 32,768 at 64; BF16 32,768 rays and 4 evaluations at width 32, 16,384 and 2 at width 64
     const int def_tail = c.bf16 ? (sdf_width >= 64 ? kRenderBf16TailRaysWide : kRenderBf16TailRays)
                                 : (sdf_width >= 64 ? kRenderBf16TailRays : kRenderTailRays);
