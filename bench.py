@@ -156,8 +156,8 @@ class ClockSampler:
 # the sources each profiled kernel is compiled from: a committed capture counts only while they are unchanged
 KERNEL_SOURCES = {
     "trace_tc_kernel": ["kns_tc.cu", "kns_tc.cuh", "kns_wave.cuh", "kns_device.cuh", "kns_kernels.h"],
-    "wave_eval_block_kernel": ["kns_wave.cu", "kns_wave.cuh", "kns_device.cuh", "kns_kernels.h"],
-    "k_tile_backward": ["kns_train_tile.cu", "kns_train.cuh", "kns_device.cuh", "kns_kernels.h"],
+    "wave_eval_warps_kernel": ["kns_wave.cu", "kns_wave.cuh", "kns_warp.cuh", "kns_device.cuh", "kns_kernels.h"],
+    "k_warp_fd_backward": ["kns_train_tile.cu", "kns_train.cuh", "kns_warp.cuh", "kns_device.cuh", "kns_kernels.h"],
 }
 
 
@@ -464,12 +464,12 @@ def run_kns(args, rank, world, local_rank):
             achieved = flops / (kms * 1e-3) / 1e12 if kms > 0 else 0.0
             t_ffma = flops / (p_ffma * 1e12) * 1e3
             t_mufu = S_ * transc / (p_mufu * 1e9) * 1e3
-            roof = {"bound": "alu", "kernel": "wave_eval_block_kernel + wave_tail_warp_kernel (FP32 evaluation class)",
+            roof = {"bound": "alu", "kernel": "wave_eval_warps_kernel + wave_tail_warp_kernel (FP32 evaluation class)",
                     "unit": "TFLOP/s", "peak": p_ffma, "achieved": achieved, "frac": achieved / p_ffma,
                     "peak_source": "measured on this GPU: FFMA micro-kernel (kns_measure_peaks), of measured",
                     "kernel_ms_per_render": kms, "flop_per_sample": 2 * mac_trace,
                     "t_floor_ms": max(t_ffma, t_mufu), "t_floor_terms_ms": {"ffma": t_ffma, "mufu": t_mufu},
-                    "traffic": profile_traffic("wave_eval_block_kernel_fp32_%s" % args.workload)}
+                    "traffic": profile_traffic("wave_eval_warps_kernel_fp32_%s" % args.workload)}
         roof["measured_peaks"] = {"ffma_tflops": p_ffma, "mufu_gops": p_mufu, "sm_count": pk["sm_count"],
                                   "hbm_gbs": hbm, "bf16_tflops": bf16_peak}
         phases = {k: st[k] for k in ("ms_generate", "ms_sort", "ms_eval_fp32", "ms_eval_bf16", "ms_shade",
@@ -501,9 +501,10 @@ def run_kns(args, rank, world, local_rank):
                           "cooperative launch), the one-warp-per-ray tail, hit count/scan/scatter, shading, FP32 "
                           "refinement")
         else:
-            launches = 4 + st["rounds"] * 5
-            launch_src = ("library round counter: gen + rounds x (scan part, scan final, scatter, eval, tail) + "
-                          "(rounds - 1) advance + hit sort (3) + shade")
+            launches = 3 + st["rounds"] * 5
+            launch_src = ("library round counter, the fewest launches it stands for: gen + rounds x (scan, scatter, "
+                          "eval, tail) + (rounds - 1) advance + hit sort (3) + shade, less the evaluation of a last "
+                          "round that is the tail's (a scan of more than 4096 keys takes two launches, not counted)")
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": max(3, args.warmup), "ms_per_step": ms_per_step, "higher_is_better": True,
                 "scaling": "weak", "vs_baseline": None, "dtype": "f32" if precision == kns.KNS_FP32 else "bf16",
@@ -855,10 +856,10 @@ def run_train(args, rank, world, local_rank):
         kms = st["ms_fd_backward"]
         achieved = flops / (kms * 1e-3) / 1e12 if kms > 0 else 0.0
         roof = {"bound": "alu", "peak": fp32_peak, "unit": "TFLOP/s",
-                "kernel": "k_tile_backward (difference points)",
+                "kernel": "k_warp_fd_backward (difference points)",
                 "peak_source": "measured on this GPU: FFMA micro-kernel (kns_measure_peaks), of measured",
                 "achieved": achieved, "frac": achieved / fp32_peak,
-                "traffic": profile_traffic("k_tile_backward_fd_train"), "algorithmic_flop_per_launch": flops,
+                "traffic": profile_traffic("k_warp_fd_backward_train"), "algorithmic_flop_per_launch": flops,
                 "kernel_ms_per_launch": kms, "flop_per_record": 2 * mac["bwd_d"],
                 "records_per_launch": st["records_fd"],
                 "note": "algorithmic work = input gradients + weight gradient; the kernel also recomputes the "

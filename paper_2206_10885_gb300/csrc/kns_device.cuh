@@ -542,8 +542,8 @@ __device__ __forceinline__ int cross_empty_box(const GridView &g, const Ray &r, 
 // voxels the walk jumps to the box's entry, or ends when the ray cannot reach the box (occ_box_entry; with the
 // field, only far from everything occupied).  Either way the voxel and parameter reached are those of the voxel walk.
 // What bounds a walk is its chain of dependent loads, one a step, and a round ends with its longest walk.  The field
-// against blocks of 8^3: 100,003 rays 0.69 -> 0.66 ms, a 511 x 383 BF16 view 2.54 -> 2.46 ms, two 1080p views of the
-// 16^3 width-32 grid 6.18 -> 6.13 ms, of the 32^3 width-64 grid 9.11 -> 8.99 ms.
+// against blocks of 8^3: 100,003 rays 0.69 -> 0.66 ms, a 511 x 383 BF16 view 2.54 -> 2.46 ms, eight 800 x 800
+// FP32 views of the 16^3 width-32 grid 6.18 -> 6.13 ms, two 1080p views of the 32^3 width-64 grid 9.11 -> 8.99 ms.
 __device__ __forceinline__ bool dda_next(const GridView &g, const Ray &r, int &vx, int &vy, int &vz, float tf,
                                          float &te) {
     const int res = g.occ_res;

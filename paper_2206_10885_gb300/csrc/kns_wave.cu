@@ -472,9 +472,9 @@ __global__ void __launch_bounds__(NT, block_min_blocks<C, BT>()) wave_eval_block
 // times while enough of them do, without a barrier: the block's warps meet only where the next tile's weights
 // replace this one's.  d is the same sum, so results do not depend on the tile shape.
 // Bound by the FMA pipe and by the rounds' serial chain: the shared tiles lost their time at a barrier per layer and
-// per pass, which every warp reached when the slowest did.  Two 1080p views of the 16^3 width-32 grid 6.64 -> 6.18 ms,
-// two of the 32^3 width-64 grid 9.67 -> 9.10 ms, four 640 x 480 views 2.16 -> 2.05 ms.  Loading the next tile's weights
-// into a second buffer gained nothing, five blocks an SM (a spill) and 16 samples a warp at width 32 were slower.
+// per pass, which every warp reached when the slowest did.  Eight 800 x 800 views of the 16^3 width-32 grid
+// 6.64 -> 6.18 ms, two 1080p views of the 32^3 width-64 grid 9.67 -> 9.10 ms, five views of 0.07 to 0.64 M rays of a
+// stack of two grids 2.16 -> 2.05 ms.  Loading the next tile's weights into a second buffer gained nothing, five blocks an SM (a spill) and 16 samples a warp at width 32 were slower.
 template <class C>
 struct EB {
     static constexpr int P = C::W == 32 ? 32 : 16, NW = 128 / P, NT = 32 * NW, BLOCKS = C::W == 32 ? 4 : 2;

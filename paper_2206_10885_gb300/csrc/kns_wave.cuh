@@ -245,7 +245,7 @@ __device__ __forceinline__ void warp_bucket_cells(const WaveArgs &a, int p, bool
 // The ends of one evaluation of a round of parity cur, for a whole warp: hits to the hit list, rays left in empty
 // voxels to the round's pending list, and rays with a next sample to the next round's queue, counts and (buckets)
 // cell buckets.  The atomics that hand out the places are issued together, by lanes 0 to 2 and the groups' first
-// lanes, so the warp waits for one round trip to L2 instead of one per list: eight 1080p views of a 32^3 width-32
+// lanes, so the warp waits for one round trip to L2 instead of one per list: eight 1080p views of a 32^3 width-64
 // grid 13.72 -> 13.56 ms, one 511 x 383 view 2.58 -> 2.54 ms.
 __device__ __forceinline__ void warp_queue(const WaveArgs &a, int cur, bool hit, bool emit, bool pend, int r, int ncell,
                                            float t_eval, bool buckets) {
