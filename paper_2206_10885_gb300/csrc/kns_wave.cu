@@ -790,15 +790,55 @@ __device__ __forceinline__ float warp_d_row(const float *__restrict__ drow, floa
     return d;
 }
 
+// The weights of its cell that a lane of the tail keeps in registers: those of the last hidden layer, at width 32 with
+// three hidden layers.  The tail is bound by its SMs' shared memory -- 92 cycles of weight reads a sample there, 46 of inputs,
+// 32 of the d row and about 43 of the copies of the cells, one for every 2.3 samples -- and the register copy saves a
+// read of 32 cycles wherever the ray stays in its cell: eight 800 x 800 views 6.09 -> 6.02 ms, 100,003 rays 0.67 ->
+// 0.66 ms.  It costs 32 registers a lane, which are free only while the slots leave no more than 16 warps an SM: with
+// two hidden layers the slots hold 24, the registers then 18 (four 64 x 64 views 0.181 -> 0.189 ms); two layers in
+// registers are slower (five views of a stack of two grids 2.01 -> 2.06 ms), and at width 64 one saves nothing.
+template <class C>
+struct TailRegs {
+    static constexpr bool LAST = C::W == 32 && C::H >= 3;
+    float last[LAST ? C::W : 1];
+
+    __device__ __forceinline__ void load(const float *wsm, int lane) {
+        if constexpr (LAST) {
+#pragma unroll
+            for (int k = 0; k < C::W; ++k) last[k] = wsm[C::tWl(C::H - 1) + k * C::W + lane];
+        }
+    }
+};
+
+// warp_layer with lane l's weights in its registers (width 32)
+__device__ __forceinline__ void warp_layer_regs(const float (&w)[32], const float *__restrict__ b, const float *in,
+                                                float *out, int lane, float beta, float inv_beta) {
+    float acc = b[lane];
+#pragma unroll
+    for (int k = 0; k < 32; k += 4) {
+        float x[4];
+        VecF<4>::load(in + k, x);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc = fmaf(w[k + c], x[c], acc);
+    }
+    out[lane] = softplus_f32(acc, beta, inv_beta);
+    __syncwarp();
+}
+
 // The SDF trace form of one sample whose encoded input row is in xin.
 template <class C>
-__device__ __forceinline__ float warp_sdf_trace(const float *__restrict__ wsm, const float *xin, float *h0, float *h1,
-                                                int lane, float beta, float inv_beta) {
+__device__ __forceinline__ float warp_sdf_trace(const float *__restrict__ wsm, const TailRegs<C> &regs, const float *xin,
+                                                float *h0, float *h1, int lane, float beta, float inv_beta) {
     warp_layer<C::INP, C::W>(wsm + C::tW0, wsm + C::tb0, xin, h0, lane, beta, inv_beta);
     float *src = h0, *dst = h1;
 #pragma unroll
     for (int l = 1; l < C::H; ++l) {
-        warp_layer<C::W, C::W>(wsm + C::tWl(l), wsm + C::tbl(l), src, dst, lane, beta, inv_beta);
+        if constexpr (TailRegs<C>::LAST) {
+            if (l == C::H - 1) warp_layer_regs(regs.last, wsm + C::tbl(l), src, dst, lane, beta, inv_beta);
+            else warp_layer<C::W, C::W>(wsm + C::tWl(l), wsm + C::tbl(l), src, dst, lane, beta, inv_beta);
+        } else {
+            warp_layer<C::W, C::W>(wsm + C::tWl(l), wsm + C::tbl(l), src, dst, lane, beta, inv_beta);
+        }
         float *tmp = src;
         src = dst;
         dst = tmp;
@@ -825,6 +865,7 @@ __global__ void __launch_bounds__(32) wave_tail_warp_kernel(GridView g, WaveArgs
     const bool cycles = a.t_hist != nullptr;
     int cached = -1;
     uint32_t phase = 0;
+    TailRegs<C> regs;
     unsigned long long nsamples = 0;
     for (;;) {
         int q = 0;
@@ -870,9 +911,10 @@ __global__ void __launch_bounds__(32) wave_tail_warp_kernel(GridView g, WaveArgs
                     return;
                 }
                 cached = cell;
+                regs.load(wsm, lane);
             }
             __syncwarp();
-            const float d = warp_sdf_trace<C>(wsm, xin, h0, h1, lane, g.beta, g.inv_beta);
+            const float d = warp_sdf_trace<C>(wsm, regs, xin, h0, h1, lane, g.beta, g.inv_beta);
             ++steps;
             ++nsamples;
             if (fabsf(d) < a.eps) {
