@@ -188,7 +188,8 @@ kns_status kns_sync(kns_ctx *ctx, void *cuda_stream, int64_t timeout_ms);
  * keeps four device copies of the weights, each in the layout one kernel family stages with bulk
  * copies (per-thread FP32, the FP32 tiles' k-major layout, the tensor-core split-BF16 layout, the
  * shading layout: about 235 KB per cell at width 64, 7.7 GB for 32^3 cells), the occupancy mask,
- * its 8^3-block mask and the index box of its occupied voxels.
+ * its 8^3-block mask, the index box of its occupied voxels and, up to 1 GiB and where it can be allocated,
+ * one byte per voxel with the distance to the nearest occupied one.
  * Errors: INVALID_ARG (NULL pointer, n_floats mismatch, N or occ_res out of range),
  * UNSUPPORTED (a width, depth or encoding the kernels are not built for), OUT_OF_MEMORY, CUDA. */
 kns_status kns_load_grid(kns_ctx *ctx, const kns_grid_desc *desc, const float *host_weights,
@@ -342,7 +343,10 @@ kns_status kns_path_trace(kns_ctx *ctx, const kns_grid *grid, const kns_camera *
 /* Batch field query (the vectorised per-cell MLP query of Sec. 3.3): for n points (device,
  * n x 3 FP32, row-major) evaluate the SDF MLP of cell m(x): sdf (device, n floats), feat (device,
  * n x feat_dim, or NULL), grad (device, n x 3 analytic input gradient, or NULL).
- * n = 0 is a successful no-op.  Errors: INVALID_ARG (NULL pts/sdf with n > 0, n < 0), CUDA. */
+ * n = 0 is a successful no-op.  Queries of 32,768 points or more, four a cell on average, are grouped by cell
+ * in stream-ordered scratch of the context's own pool (about 24 bytes a point, at most 128 MB kept between
+ * calls), or answered point by point where that cannot be allocated.
+ * Errors: INVALID_ARG (NULL pts/sdf with n > 0, n < 0), CUDA. */
 kns_status kns_sdf(kns_ctx *ctx, const kns_grid *grid, const float *pts, int64_t n, float *sdf,
                    float *feat, float *grad, void *cuda_stream);
 

@@ -58,7 +58,8 @@ struct Cfg {
 };
 
 constexpr int kOccDist = 15;         // the largest distance the field tells apart
-constexpr size_t kOccDistBytes = (size_t)1 << 30;  // a grid whose field would be larger does without
+constexpr size_t kOccDistBytes = (size_t)1 << 30;  // a grid whose field would be larger keeps none (for its
+                                                   // memory; the walk is faster with one at any size)
 
 // Everything a kernel needs to read a resident grid (passed by value).
 struct GridView {
