@@ -185,7 +185,7 @@ cudaError_t launch_tiles(const GridView &g, const PointsScratch &sc, int64_t n, 
                          int sm_count, cudaStream_t s) {
     constexpr int smem = PWARPS * PL<C>::ROWS * row_stride(P) * (int)sizeof(float);
     static_assert(smem <= 200 * 1024, "point tiles do not fit in shared memory");
-    static std::atomic<int> per_sm{0};
+    static PerDevice per_sm;
     int nb = 0;
     cudaError_t e = resident_blocks(points_tile_kernel<C, P>, 32 * PWARPS, smem, per_sm, nb);
     if (e != cudaSuccess) return e;

@@ -689,14 +689,16 @@ cudaError_t launch_wave_eval_tc_cfg(const GridView &g, const WaveArgs &a, int cu
     // Resident blocks per SM from the kernel's own resources (registers, shared memory, threads) and the
     // tensor memory (accumulator and activation columns, of 512 per SM).  The occupancy query is not used here: it reports one
     // block per SM for every kernel that allocates tensor memory.
-    static std::atomic<int> per_sm{0};
-    int nb = per_sm.load();
+    static PerDevice per_sm;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    int nb = per_sm.get(dev);
     if (nb <= 0) {
-        cudaError_t e = cudaFuncSetAttribute(wave_eval_tc_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
+        e = cudaFuncSetAttribute(wave_eval_tc_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
         cudaFuncAttributes fa{};
-        int dev = 0, smem_sm = 0, reserved = 0, regs_sm = 0;
+        int smem_sm = 0, reserved = 0, regs_sm = 0;
         if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, wave_eval_tc_kernel<C>);
-        if (e == cudaSuccess) e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
@@ -705,7 +707,7 @@ cudaError_t launch_wave_eval_tc_cfg(const GridView &g, const WaveArgs &a, int cu
         const int by_regs = regs_sm / (regs_warp * 4);
         const int by_smem = smem_sm / (T::SMEM + (int)fa.sharedSizeBytes + reserved);
         nb = std::max(1, std::min(std::min(by_regs, by_smem), std::min(16, 512 / (int)pow2_cols(T::TCOLS))));
-        per_sm.store(nb);
+        per_sm.set(dev, nb);
     }
     wave_eval_tc_kernel<C><<<sm_count * nb, 128, T::SMEM, s>>>(g, a, cur);
     return cudaGetLastError();

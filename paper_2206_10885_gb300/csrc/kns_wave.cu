@@ -1113,7 +1113,7 @@ template <class C, int BT, int NT>
 cudaError_t launch_block_eval(const GridView &g, const WaveArgs &a, int cur, int sm_count, cudaStream_t s) {
     constexpr int smem = block_eval_smem_bytes<C, BT>();
     static_assert(smem <= 220 * 1024, "block tile does not fit in shared memory");
-    static std::atomic<int> per_sm{0};
+    static PerDevice per_sm;
     int nb = 0;
     cudaError_t e = resident_blocks(wave_eval_block_kernel<C, BT, NT>, NT, smem, per_sm, nb);
     if (e != cudaSuccess) return e;
@@ -1124,7 +1124,7 @@ cudaError_t launch_block_eval(const GridView &g, const WaveArgs &a, int cur, int
 template <class C>
 cudaError_t launch_warps_eval(const GridView &g, const WaveArgs &a, int cur, int sm_count, cudaStream_t s) {
     using B = EB<C>;
-    static std::atomic<int> single{0}, stack{0};
+    static PerDevice single, stack;
     int nb = 0;
     cudaError_t e = g.sub_boxes ? resident_blocks(wave_eval_warps_kernel<C, true>, B::NT, B::SMEM, stack, nb)
                                 : resident_blocks(wave_eval_warps_kernel<C, false>, B::NT, B::SMEM, single, nb);
@@ -1161,7 +1161,7 @@ cudaError_t launch_wave_tail_cfg(const GridView &g, const WaveArgs &a, int cur, 
     // one-warp blocks, as many as fit on the SMs at once (each holds one cell's weights)
     constexpr int tsmem = tail_smem_floats<C>() * (int)sizeof(float);
     static_assert(tsmem <= 64 * 1024, "tail weight slot does not fit");
-    static std::atomic<int> tail_per_sm{0};
+    static PerDevice tail_per_sm;
     int tail_blocks = 0;
     cudaError_t e = resident_blocks(wave_tail_warp_kernel<C, false>, 32, tsmem, tail_per_sm, tail_blocks);
     if (e != cudaSuccess) return e;

@@ -11,10 +11,9 @@
 // Hits are shaded after the last wave (normal from the analytic gradient, colour MLP of Eq. 3).
 #pragma once
 
-#include <atomic>
-
 #include "kns_device.cuh"
 #include "kns_kernels.h"
+#include "kns_launch.h"
 
 namespace kns {
 
@@ -375,22 +374,6 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
-}
-
-// Resident blocks per SM of a kernel with `smem` bytes of dynamic shared memory (registers and shared
-// memory both count), after allowing it the largest shared-memory carve-out; asked once per kernel.
-template <class K>
-cudaError_t resident_blocks(K kernel, int threads, int smem, std::atomic<int> &cache, int &out) {
-    out = cache.load();
-    if (out > 0) return cudaSuccess;
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100)) != cudaSuccess ||
-        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&out, kernel, threads, smem)) != cudaSuccess)
-        return e;
-    if (out < 1) out = 1;
-    cache.store(out);
-    return cudaSuccess;
 }
 
 }  // namespace kns
