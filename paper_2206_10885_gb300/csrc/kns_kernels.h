@@ -35,6 +35,7 @@ struct WaveCtrl {
     int tail_parity;                  // queue parity of the round it left to the one-warp-per-ray tail
     int n_list[2];                    // by parity: tiles listed for the round while its samples were queued ...
     int over[2];                      // ... and whether a cell held more than kBucket samples
+    int handover;                     // the round at hand is the tail's (decided by the last block out of the one before)
     int round_live[512];              // samples queued for each round
     int round_tiles[512];             // tiles of each round (persistent BF16 trace)
     unsigned long long round_end_ns[512];  // global timer at the end of each round

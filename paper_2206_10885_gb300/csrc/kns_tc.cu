@@ -516,8 +516,9 @@ __global__ void __launch_bounds__(NW * 128, 1) trace_tc_kernel(GridView g, WaveA
     for (;; ++round) {
         const int cur = round & 1, nxt = cur ^ 1;
         // a round of at most tail_rays rays (after the first) is finished one warp per ray in FP32
-        // (wave_tail_warp_kernel, launched after this kernel): it is sorted and scattered, then the loop ends
-        const bool handover = round > 0 && ctrl->n_live[cur] + ctrl->n_pend[nxt] <= a.tail_max;
+        // (wave_tail_warp_kernel, launched after this kernel): it is sorted and scattered, then the loop ends.  The
+        // counts are not compared here: the first blocks to walk pending rays add to them
+        const bool handover = ctrl->handover != 0;
         if (handover) {
             // the rays the previous round left in empty voxels walk to their next occupied voxel first
             // and join this round, which the tail then finishes
@@ -659,8 +660,13 @@ __global__ void __launch_bounds__(NW * 128, 1) trace_tc_kernel(GridView g, WaveA
                 advance_pending(g, a, nxt, nxt, b + (tid & 31), n, to_buckets);
             }
         }
-        // the counters the next round adds to, which this one has finished with, are reset before any block goes on
+        // the counters the next round adds to, which this one has finished with, are reset and the hand-over is decided
+        // before any block goes on (half a microsecond a round, which a render that never hands over is spared)
         if (!(ok = grid_sync(ctrl, gen, &s_flag, kGridPolls, [&]() {
+                  if (a.tail_max > 0) {
+                      asm volatile("fence.acq_rel.gpu;" ::: "memory");  // every block's counts
+                      ctrl->handover = __ldcg(&ctrl->n_live[nxt]) + __ldcg(&ctrl->n_pend[cur]) <= a.tail_max ? 1 : 0;
+                  }
                   ctrl->round_live[round] = ctrl->n_live[cur];
                   ctrl->n_live[cur] = ctrl->n_pend[nxt] = ctrl->n_list[cur] = ctrl->over[cur] = 0;
                   ctrl->next_tile_bf = ctrl->next_adv = 0;
