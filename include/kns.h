@@ -26,6 +26,13 @@
  *  - Memory: the caller owns every input and output buffer and passes plain
  *    pointers (device pointers unless stated "host").  The library never
  *    frees caller memory.  Grids own the device copies of their weights.
+ *    A context keeps its scratch between calls: about 89 bytes per ray of
+ *    its largest render, 56 per cell and, once it has rendered in KNS_BF16,
+ *    4.1 KB per cell for rounds that need no sort (135 MB for 32^3 cells,
+ *    1.1 GB for 64^3).  The latter, a grid's distance field and the scratch
+ *    of large field queries are taken only where there is room: without them
+ *    results are the same and calls slower, a context out of memory gives its
+ *    own back before it reports so, and does not ask for it on every call.
  *  - Threads: a context may be used from several host threads; calls on one
  *    context are serialised on the host.  Their GPU work shares the context's
  *    scratch, so one context's renders must also be ordered on the GPU: issue
@@ -285,6 +292,11 @@ kns_status kns_measure_peaks(kns_ctx *ctx, void *cuda_stream, kns_peaks *out);
  * record KNS_ERR_TIMEOUT in the context's status word (returned and cleared by the next kns_sync) and
  * return; the context stays usable.  Errors: INVALID_ARG (which not 0 or 1), CUDA. */
 kns_status kns_selftest_timeout(kns_ctx *ctx, int32_t which, void *cuda_stream);
+
+/* Self-test of the paths without the memory that the library can do without (not part of the method): gives back
+ * what the context holds of it and refuses later requests above max_bytes (< 0: none) as if the device were full.
+ * *refused (may be NULL) receives the number of requests refused or failed so far.  Errors: INVALID_ARG (NULL ctx). */
+kns_status kns_selftest_memory(kns_ctx *ctx, int64_t max_bytes, int64_t *refused);
 
 /* One view of a multi-view render: camera, image size, its own output buffers (device pointers for
  * W*H pixels, layout as kns_frame) and which grid of a stack it renders (0 for a single grid; its

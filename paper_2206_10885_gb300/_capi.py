@@ -155,6 +155,8 @@ def lib():
             L.kns_measure_peaks.restype = st
             L.kns_selftest_timeout.argtypes = [vp, C.c_int32, vp]
             L.kns_selftest_timeout.restype = st
+            L.kns_selftest_memory.argtypes = [vp, C.c_int64, C.POINTER(C.c_int64)]
+            L.kns_selftest_memory.restype = st
             L.kns_get_round_trace.argtypes = [vp, C.POINTER(kns_round_info), C.c_int32, C.POINTER(C.c_int32)]
             L.kns_get_round_trace.restype = st
             L.kns_trace_rays.argtypes = [vp, vp, vp, vp, C.c_int64, C.c_int, C.c_float, C.POINTER(kns_frame),
@@ -301,6 +303,13 @@ def kns_get_round_trace(ctx: int, max_rounds: int = 1024) -> list:
 def kns_selftest_timeout(ctx: int, which: int, stream: int = 0) -> None:
     """Runs a device wait that nothing satisfies (0: mbarrier, 1: grid barrier); the next sync reports it."""
     _check(lib().kns_selftest_timeout(ctx, which, stream), ctx)
+
+
+def kns_selftest_memory(ctx: int, max_bytes: int) -> int:
+    """Refuses the context memory it can do without above max_bytes (< 0: no bound); the requests refused so far."""
+    n = C.c_int64(0)
+    _check(lib().kns_selftest_memory(ctx, max_bytes, C.byref(n)), ctx)
+    return n.value
 
 
 def kns_sdf(ctx: int, grid: int, pts_ptr: int, n: int, sdf_ptr: int, feat_ptr: int = None, grad_ptr: int = None,

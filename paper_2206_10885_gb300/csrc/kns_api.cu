@@ -29,6 +29,7 @@ struct WaveScratch {
     int *cellbuf = nullptr;  // count[2], fill[2], off, tile_off (6 * (nc + 1) ints)
     int *buckets = nullptr;  // persistent BF16 trace: bucket[2], list[2], taken (kns_kernels.h)
     int bucket_nc = 0;       // cells they are sized for
+    int bucket_refused = 0;  // cells there was no memory for (0: not asked): not asked again for as many
     int4 *tiles = nullptr;   // tile descriptors of a round (max_tiles(rays, 2 nc))
     int *pend_r[2] = {nullptr, nullptr};  // per round parity: rays waiting for the occupancy DDA
     float *pend_t[2] = {nullptr, nullptr};
@@ -96,6 +97,9 @@ struct kns_ctx {
     int round0 = 0;                        // its last batch's first round
     // stream-ordered scratch of grouped field queries: calls on several streams each get their own
     cudaMemPool_t pool = nullptr;
+    // memory the context can do without (cell buckets, a grid's distance field, a field query's scratch)
+    int64_t spare_max = INT64_MAX;         // the most that one of these may take (kns_selftest_memory)
+    int64_t spare_refused = 0;             // requests that were refused or failed
 };
 
 struct kns_grid {
@@ -137,6 +141,7 @@ kns_status set_err(kns_ctx *ctx, kns_status st, const char *fmt, ...) {
 }
 
 kns_status cuda_err(kns_ctx *ctx, cudaError_t e, const char *what) {
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();  // reported here: the next launch's check is its own
     return set_err(ctx, e == cudaErrorMemoryAllocation ? KNS_ERR_OUT_OF_MEMORY : KNS_ERR_CUDA, "%s: %s (%s)", what,
                    cudaGetErrorString(e), cudaGetErrorName(e));
 }
@@ -381,6 +386,38 @@ void free_scratch(WaveScratch &w) {
     cudaFree(w.d_views);
     cudaFree(w.ctrl);
     w = WaveScratch{};
+}
+
+// Device memory the caller can do without: NULL, and no error, where it cannot be had.
+template <class T>
+T *spare_alloc(kns_ctx *ctx, size_t bytes) {
+    T *p = nullptr;
+    if ((int64_t)bytes <= ctx->spare_max && cudaMalloc((void **)&p, bytes) == cudaSuccess) return p;
+    cudaGetLastError();
+    ++ctx->spare_refused;
+    return nullptr;
+}
+
+// Gives back what the context holds and can do without; false where that is nothing.
+bool give_back(kns_ctx *ctx) {
+    WaveScratch &w = ctx->ws;
+    uint64_t kept = 0;
+    if (ctx->pool) cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &kept);
+    if (!w.buckets && kept == 0) return false;
+    cudaDeviceSynchronize();  // earlier calls may still use it
+    cudaFree(w.buckets);
+    w.buckets = nullptr;
+    w.bucket_nc = 0;
+    if (ctx->pool) cudaMemPoolTrimTo(ctx->pool, 0);
+    cudaGetLastError();
+    return true;
+}
+
+// f(), and once more with that memory given back where f ran out of memory.
+template <class F>
+kns_status with_room(kns_ctx *ctx, F f) {
+    const kns_status st = f();
+    return st == KNS_ERR_OUT_OF_MEMORY && give_back(ctx) ? f() : st;
 }
 
 // Render tiling: samples per tile (a warp tile, or a 256-thread block tile).
@@ -733,9 +770,10 @@ kns_status kns_sync(kns_ctx *ctx, void *cuda_stream, int64_t timeout_ms) {
 
 // Uploads n_sub grids of one descriptor as one resident object (n_sub = 1: a single grid): their cells
 // are numbered back to back (grid k's cell c is k N^3 + c) in every weight layout, and their occupancy
-// masks and 8^3-block masks follow each other, each built from its own grid's SDF.
+// masks and 8^3-block masks follow each other, each built from its own grid's SDF.  `field`: with the distance field
+// of the masks, where there is room for it.
 static kns_status load_grid_impl(kns_ctx *ctx, const kns_grid_desc *desc, const float *host_weights,
-                                 size_t n_floats, int n_sub, const uint64_t *occ_words, kns_grid **out) {
+                                 size_t n_floats, int n_sub, const uint64_t *occ_words, bool field, kns_grid **out) {
     if (!desc || !host_weights || !out) return set_err(ctx, KNS_ERR_INVALID_ARG, "NULL desc, weights or out");
     *out = nullptr;
     kns_status st = check_desc(ctx, *desc);
@@ -825,11 +863,13 @@ static kns_status load_grid_impl(kns_ctx *ctx, const kns_grid_desc *desc, const 
         // the distance field and a buffer to build it in; without the memory for them the walk uses the block mask
         uint8_t *dist_tmp = nullptr;
         const size_t nvox = (size_t)d.occ_res * d.occ_res * d.occ_res;
-        if (e == cudaSuccess && nvox * (size_t)n_sub <= kns::kOccDistBytes &&
-            (cudaMalloc(&g->d_dist, nvox * (size_t)n_sub) != cudaSuccess || cudaMalloc(&dist_tmp, nvox) != cudaSuccess)) {
-            cudaGetLastError();
-            cudaFree(g->d_dist);
-            g->d_dist = nullptr;
+        if (e == cudaSuccess && field && nvox * (size_t)n_sub <= kns::kOccDistBytes) {
+            g->d_dist = spare_alloc<uint8_t>(ctx, nvox * (size_t)n_sub);
+            if (g->d_dist) dist_tmp = spare_alloc<uint8_t>(ctx, nvox);
+            if (!dist_tmp) {
+                cudaFree(g->d_dist);
+                g->d_dist = nullptr;
+            }
         }
         fill_view(g);
         float diag = 0.f;
@@ -895,18 +935,25 @@ static kns_status load_grid_impl(kns_ctx *ctx, const kns_grid_desc *desc, const 
     return KNS_OK;
 }
 
+static kns_status load_grid_in(kns_ctx *ctx, const kns_grid_desc *desc, const float *host_weights, size_t n_floats,
+                               int n_sub, const uint64_t *occ_words, kns_grid **out) {
+    kns_status st = with_room(ctx, [&] { return load_grid_impl(ctx, desc, host_weights, n_floats, n_sub, occ_words, true, out); });
+    if (st == KNS_ERR_OUT_OF_MEMORY) st = load_grid_impl(ctx, desc, host_weights, n_floats, n_sub, occ_words, false, out);
+    return st;
+}
+
 kns_status kns_load_grid(kns_ctx *ctx, const kns_grid_desc *desc, const float *host_weights, size_t n_floats,
                          const uint64_t *occ_words, kns_grid **out) {
     if (!ctx) return KNS_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> lk(ctx->mu);
-    return load_grid_impl(ctx, desc, host_weights, n_floats, 1, occ_words, out);
+    return load_grid_in(ctx, desc, host_weights, n_floats, 1, occ_words, out);
 }
 
 kns_status kns_load_grid_stack(kns_ctx *ctx, const kns_grid_desc *desc, int32_t n_grids, const float *host_weights,
                                size_t n_floats, const uint64_t *occ_words, kns_grid **out) {
     if (!ctx) return KNS_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> lk(ctx->mu);
-    return load_grid_impl(ctx, desc, host_weights, n_floats, n_grids, occ_words, out);
+    return load_grid_in(ctx, desc, host_weights, n_floats, n_grids, occ_words, out);
 }
 
 kns_status kns_grid_stack_size(const kns_grid *grid, int32_t *n_grids) {
@@ -986,6 +1033,7 @@ void kns_free_grid(kns_grid *g) {
         cudaFree(g->d_occ_coarse);
         cudaFree(g->d_dist);
         cudaFree(g->d_boxes);
+        g->ctx->ws.bucket_refused = 0;  // there may be room now
     }
     delete g;
 }
@@ -1091,7 +1139,7 @@ kns_status render_views_impl(kns_ctx *ctx, const kns_grid *grid, const std::vect
     const int NC = grid->n_sub * grid->desc.N * grid->desc.N * grid->desc.N;  // every grid of a stack
     const int nkeys = NC;  // sort keys: cells
     const int nv = (int)views.size();
-    kns_status st = ensure_scratch(ctx, rays, nkeys, nv);
+    kns_status st = with_room(ctx, [&] { return ensure_scratch(ctx, rays, nkeys, nv); });
     if (st != KNS_OK) return st;
     WaveScratch &w = ctx->ws;
     int max_W = 0, max_H = 0;
@@ -1159,15 +1207,18 @@ kns_status render_views_impl(kns_ctx *ctx, const kns_grid *grid, const std::vect
     a.ctrl = w.ctrl;
     if (cfg.bf16 && cfg.persistent) {
         const size_t per = (size_t)(2 * kns::kBucket) * nkeys, lists = (size_t)2 * (kns::kBucket / 128) * nkeys;
-        if (w.bucket_nc < nkeys) {  // without them (no memory left) every round is sorted
-            cudaDeviceSynchronize();
-            cudaFree(w.buckets);
-            w.buckets = nullptr;
-            w.bucket_nc = 0;
-            if (cudaMalloc((void **)&w.buckets, sizeof(int) * (per + lists + nkeys)) == cudaSuccess) w.bucket_nc = nkeys;
-            else cudaGetLastError();
+        // without them (no memory left) every round is sorted; what was refused is not asked for on every render
+        if (w.bucket_nc < nkeys && (w.bucket_refused == 0 || nkeys < w.bucket_refused)) {
+            if (w.buckets) {
+                cudaDeviceSynchronize();  // an earlier render may still use them
+                cudaFree(w.buckets);
+                w.bucket_nc = 0;
+            }
+            w.buckets = spare_alloc<int>(ctx, sizeof(int) * (per + lists + nkeys));
+            if (w.buckets) w.bucket_nc = nkeys;
+            else w.bucket_refused = nkeys;
         }
-        if (w.buckets) {
+        if (w.bucket_nc >= nkeys) {
             for (int p = 0; p < 2; ++p) {
                 a.bucket[p] = w.buckets + p * (per / 2);
                 a.list[p] = w.buckets + per + p * (lists / 2);
@@ -1440,7 +1491,7 @@ kns_status kns_path_trace(kns_ctx *ctx, const kns_grid *grid, const kns_camera *
     kns_status st = resolve_opts(ctx, opts, eps, cfg, grid->desc.sdf_width);
     if (st != KNS_OK) return st;
     DeviceScope ds(ctx->device);
-    if ((st = ensure_pt_scratch(ctx, n, n_cams)) != KNS_OK) return st;
+    if ((st = with_room(ctx, [&] { return ensure_pt_scratch(ctx, n, n_cams); })) != KNS_OK) return st;
     PtScratch &p = ctx->ps;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     kns::PtArgs a{};
@@ -1551,6 +1602,17 @@ kns_status kns_selftest_timeout(kns_ctx *ctx, int32_t which, void *cuda_stream) 
     return KNS_OK;
 }
 
+kns_status kns_selftest_memory(kns_ctx *ctx, int64_t max_bytes, int64_t *refused) {
+    if (!ctx) return KNS_ERR_INVALID_ARG;
+    std::lock_guard<std::mutex> lk(ctx->mu);
+    DeviceScope ds(ctx->device);
+    give_back(ctx);
+    ctx->ws.bucket_refused = 0;
+    ctx->spare_max = max_bytes < 0 ? INT64_MAX : max_bytes;
+    if (refused) *refused = ctx->spare_refused;
+    return KNS_OK;
+}
+
 kns_status kns_get_round_trace(kns_ctx *ctx, kns_round_info *out, int32_t max_rounds, int32_t *n_rounds) {
     if (!ctx) return KNS_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> lk(ctx->mu);
@@ -1617,8 +1679,10 @@ static cudaError_t points_grouped(kns_ctx *ctx, const kns_grid *grid, const floa
                  b_sorted = up(sizeof(float4) * (size_t)n),
                  b_tiles = up(sizeof(int4) * (size_t)kns::points_max_tiles(n, g.ncl));
     unsigned char *p = nullptr;
-    if (cudaMallocFromPoolAsync((void **)&p, b_ctl + b_rank + b_sorted + b_tiles, ctx->pool, s) != cudaSuccess) {
+    if ((int64_t)(b_ctl + b_rank + b_sorted + b_tiles) > ctx->spare_max ||
+        cudaMallocFromPoolAsync((void **)&p, b_ctl + b_rank + b_sorted + b_tiles, ctx->pool, s) != cudaSuccess) {
         cudaGetLastError();
+        ++ctx->spare_refused;
         return cudaSuccess;
     }
     grouped = true;
@@ -1824,7 +1888,8 @@ kns_status kns_train_forward(kns_ctx *ctx, const kns_grid_desc *desc, const floa
     const int S = b.n_strat + b.n_imp;
     const int NC = desc->N * desc->N * desc->N;
     ctx->ts.pending = false;
-    if ((st = ensure_train_scratch(ctx, b.n_rays, S, b.n_strat, b.n_eik, 2 * NC)) != KNS_OK) return st;
+    if ((st = with_room(ctx, [&] { return ensure_train_scratch(ctx, b.n_rays, S, b.n_strat, b.n_eik, 2 * NC); })) != KNS_OK)
+        return st;
     TrainScratch &t = ctx->ts;
     kns::TrainArgs a{};
     a.N = desc->N;
