@@ -1205,7 +1205,7 @@ kns_status render_views_impl(kns_ctx *ctx, const kns_grid *grid, const std::vect
     a.off = w.cellbuf + 4 * (nkeys + 1);
     a.tile_off = w.cellbuf + 5 * (nkeys + 1);
     a.ctrl = w.ctrl;
-    if (cfg.bf16 && cfg.persistent) {
+    if (cfg.bf16 && cfg.persistent && rays > cfg.tail_rays) {  // (fewer: the tail takes the second round)
         const size_t per = (size_t)(2 * kns::kBucket) * nkeys, lists = (size_t)2 * (kns::kBucket / 128) * nkeys;
         // without them (no memory left) every round is sorted; what was refused is not asked for on every render
         if (w.bucket_nc < nkeys && (w.bucket_refused == 0 || nkeys < w.bucket_refused)) {

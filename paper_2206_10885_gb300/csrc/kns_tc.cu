@@ -527,7 +527,10 @@ __global__ void __launch_bounds__(NW * 128, 1) trace_tc_kernel(GridView g, WaveA
                 advance_pending(g, a, nxt, cur, i, n);
             if (!(ok = grid_sync(ctrl, gen, &s_flag))) break;
         }
-        const bool to_buckets = a.bucket[0] && ctrl->n_live[cur] <= kBucketRays;
+        // (a first round of no more rays than the tail takes has no successor here that would use them: filling them cost
+        // a 24 x 16 view 14 of 250 us)
+        const bool to_buckets = a.bucket[0] && ctrl->n_live[cur] <= kBucketRays &&
+                                ctrl->n_live[cur] + ctrl->n_pend[nxt] > a.tail_max;
         const bool from_buckets = queued && !handover && !ctrl->over[cur];
         queued = to_buckets;
         if (from_buckets) {

@@ -79,3 +79,17 @@ def test_bf16_rounds_without_buckets(kns):
     for out in outs:
         for k in ref:
             assert torch.equal(out[k], ref[k]), k
+
+
+@pytest.mark.parametrize("tail,asked", [(-1, 1), (63, 1), (64, 0), (0, 0)])
+def test_a_render_of_no_more_rays_than_the_tail_takes_wants_no_buckets(kns, tail, asked):
+    """Its second round is the tail's (tail 0: the default limit, 32,768 rays)."""
+    desc = S.GridDesc(N=2, sdf_hidden=2, sdf_width=32, col_width=32)
+    with kns.Context(0) as ctx:
+        kns.capi.kns_selftest_memory(ctx.handle, 0)
+        grid = kns.Grid.load(ctx, desc, S.sal_sphere_grid(desc, seed=5))
+        kns.render(ctx, grid, S.orbit_cameras(1, 8, 8, seed=3), 8, 8, 64, 1e-4, precision=kns.KNS_BF16,
+                   tuning=dict(tail_rays=tail))
+        ctx.sync()
+        assert kns.capi.kns_selftest_memory(ctx.handle, -1) == asked
+        grid.free()
