@@ -518,20 +518,21 @@ __global__ void __launch_bounds__(NW * 128, 1) trace_tc_kernel(GridView g, WaveA
         // a round of at most tail_rays rays (after the first) is finished one warp per ray in FP32
         // (wave_tail_warp_kernel, launched after this kernel): it is sorted and scattered, then the loop ends.  The
         // counts are not compared here: the first blocks to walk pending rays add to them
-        const bool handover = ctrl->handover != 0;
+        // (the round's words are read together, in one round trip to L2)
+        const bool handover = ctrl->handover != 0, over = ctrl->over[cur] != 0;
+        const int live = ctrl->n_live[cur], pending = ctrl->n_pend[nxt];
         if (handover) {
             // the rays the previous round left in empty voxels walk to their next occupied voxel first
             // and join this round, which the tail then finishes
-            const int n = ctrl->n_pend[nxt], bound = (n + 31) & ~31;
+            const int bound = (pending + 31) & ~31;
             for (int i = blockIdx.x * blockDim.x + tid; i < bound; i += gridDim.x * blockDim.x)
-                advance_pending(g, a, nxt, cur, i, n);
+                advance_pending(g, a, nxt, cur, i, pending);
             if (!(ok = grid_sync(ctrl, gen, &s_flag))) break;
         }
         // (a first round of no more rays than the tail takes has no successor here that would use them: filling them cost
         // a 24 x 16 view 14 of 250 us)
-        const bool to_buckets = a.bucket[0] && ctrl->n_live[cur] <= kBucketRays &&
-                                ctrl->n_live[cur] + ctrl->n_pend[nxt] > a.tail_max;
-        const bool from_buckets = queued && !handover && !ctrl->over[cur];
+        const bool to_buckets = a.bucket[0] && live <= kBucketRays && live + pending > a.tail_max;
+        const bool from_buckets = queued && !handover && !over;
         queued = to_buckets;
         if (from_buckets) {
             if (blockIdx.x == 0 && tid == 0) {
@@ -654,13 +655,12 @@ __global__ void __launch_bounds__(NW * 128, 1) trace_tc_kernel(GridView g, WaveA
                 w.n_eval = 0;
                 break;
             }
-            const int n = ctrl->n_pend[nxt];
             for (;;) {
                 int b = 0;
                 if ((tid & 31) == 0) b = atomicAdd(&ctrl->next_adv, 32);
                 b = __shfl_sync(FULL, b, 0);
-                if (b >= n) break;
-                advance_pending(g, a, nxt, nxt, b + (tid & 31), n, to_buckets);
+                if (b >= pending) break;
+                advance_pending(g, a, nxt, nxt, b + (tid & 31), pending, to_buckets);
             }
         }
         // the counters the next round adds to, which this one has finished with, are reset and the hand-over is decided
