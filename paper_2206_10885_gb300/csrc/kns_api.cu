@@ -1676,11 +1676,10 @@ static cudaError_t points_grouped(kns_ctx *ctx, const kns_grid *grid, const floa
     }
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t b_ctl = up(sizeof(int) * (2 + (size_t)g.ncl)), b_rank = up(sizeof(int) * (size_t)n),
-                 b_sorted = up(sizeof(float4) * (size_t)n),
-                 b_tiles = up(sizeof(int4) * (size_t)kns::points_max_tiles(n, g.ncl));
+                 b_sorted = up(sizeof(float4) * (size_t)n), b_seg = up(sizeof(int4) * (size_t)g.ncl),
+                 bytes = b_ctl + b_rank + b_sorted + b_seg + up(sizeof(int4) * (size_t)kns::points_max_tiles(n, g.ncl));
     unsigned char *p = nullptr;
-    if ((int64_t)(b_ctl + b_rank + b_sorted + b_tiles) > ctx->spare_max ||
-        cudaMallocFromPoolAsync((void **)&p, b_ctl + b_rank + b_sorted + b_tiles, ctx->pool, s) != cudaSuccess) {
+    if ((int64_t)bytes > ctx->spare_max || cudaMallocFromPoolAsync((void **)&p, bytes, ctx->pool, s) != cudaSuccess) {
         cudaGetLastError();
         ++ctx->spare_refused;
         return cudaSuccess;
@@ -1691,7 +1690,8 @@ static cudaError_t points_grouped(kns_ctx *ctx, const kns_grid *grid, const floa
     sc.count = sc.ctl + 2;
     sc.rank = (int *)(p + b_ctl);
     sc.sorted = (float4 *)(p + b_ctl + b_rank);
-    sc.tiles = (int4 *)(p + b_ctl + b_rank + b_sorted);
+    sc.seg = (int4 *)(p + b_ctl + b_rank + b_sorted);
+    sc.tiles = (int4 *)(p + b_ctl + b_rank + b_sorted + b_seg);
     cudaError_t e = kns::launch_points_sort(g, pts, (int)n, sc, ctx->sm_count, s);
     if (e == cudaSuccess) e = kns::launch_points_tiles(grid->shape, g, sc, n, sdf, feat, grad, ctx->sm_count, s);
     const cudaError_t ef = cudaFreeAsync(p, s);

@@ -139,7 +139,8 @@ constexpr int kPointsTile = 16;                // points per tile
 constexpr int64_t kPointsChunk = 1 << 22;      // points grouped at a time
 struct PointsScratch {
     int *ctl;        // points placed, tiles made; the cells' counts follow
-    int *count;      // per cell: its points, then the start of its segment
+    int *count;      // per cell: its points
+    int4 *seg;       // per cell that has points: its segment's start, its first tile, its points
     int *rank;       // per point: its place in its cell
     float4 *sorted;  // x, y, z, point number (bit pattern), by cell
     int4 *tiles;     // cell, first sorted point, points

@@ -324,9 +324,11 @@ cudaError_t launch_wave_scatter(const WaveArgs &a, int cur, int blocks, cudaStre
 }
 
 // ---------------------------------------------------------------- field-query points by cell
-// Three passes: a count per cell (each point keeps its rank in its cell), a segment of `sorted` and tiles of
-// `tile` points for every non-empty cell, and the scatter.  The segments lie in any order, so the blocks of
-// the second pass only add their totals to two cursors.  Bound by the points' 12 bytes, read twice.
+// Three passes: a count per cell (each point keeps its rank in its cell), a segment of `sorted` and a run of tiles of
+// `tile` points for every non-empty cell, and the scatter, in which the first point of each tile also writes its
+// descriptor (one thread per cell writing all of them took 0.5 ms for a million points in one cell).  The segments lie
+// in any order, so the blocks of the second pass only add their totals to two cursors.  Bound by the points' 12
+// bytes, read twice.
 __global__ void __launch_bounds__(256) points_count_kernel(GridView g, const float *__restrict__ pts, int n,
                                                            PointsScratch s) {
     const int lane = threadIdx.x & 31, bound = (n + 31) & ~31;
@@ -356,17 +358,17 @@ __global__ void __launch_bounds__(SCAN_THREADS) points_segment_kernel(PointsScra
     }
     __syncthreads();
     if (n == 0) return;
-    const int first = base[0] + incl_n - n;
-    int t = base[1] + incl_t - nt;
-    s.count[c] = first;  // the scatter's segment starts
-    for (int i = 0; i < n; i += tile) s.tiles[t++] = make_int4(c, first + i, min(tile, n - i), 0);
+    s.seg[c] = make_int4(base[0] + incl_n - n, base[1] + incl_t - nt, n, 0);
 }
 
 __global__ void __launch_bounds__(256) points_scatter_kernel(GridView g, const float *__restrict__ pts, int n,
-                                                             PointsScratch s) {
+                                                             PointsScratch s, int tile) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float x = pts[3 * (int64_t)i], y = pts[3 * (int64_t)i + 1], z = pts[3 * (int64_t)i + 2];
-        s.sorted[s.count[cell_of(g, x, y, z)] + s.rank[i]] = make_float4(x, y, z, __int_as_float(i));
+        const int c = cell_of(g, x, y, z), r = s.rank[i];
+        const int4 seg = s.seg[c];
+        s.sorted[seg.x + r] = make_float4(x, y, z, __int_as_float(i));
+        if (r % tile == 0) s.tiles[seg.y + r / tile] = make_int4(c, seg.x + r, min(tile, seg.z - r), 0);
     }
 }
 
@@ -377,7 +379,7 @@ cudaError_t launch_points_sort(const GridView &g, const float *pts, int n, const
     const int blocks = std::min(sm_count * 8, (n + 255) / 256);
     points_count_kernel<<<blocks, 256, 0, s>>>(g, pts, n, sc);
     points_segment_kernel<<<(g.ncl + SCAN_THREADS - 1) / SCAN_THREADS, SCAN_THREADS, 0, s>>>(sc, g.ncl, kPointsTile);
-    points_scatter_kernel<<<blocks, 256, 0, s>>>(g, pts, n, sc);
+    points_scatter_kernel<<<blocks, 256, 0, s>>>(g, pts, n, sc, kPointsTile);
     return cudaGetLastError();
 }
 
