@@ -704,6 +704,15 @@ kns_status kns_create(int device, kns_ctx **out) {
         delete c;
         return cuda_err(nullptr, e, "context events and stream");
     }
+    // the field queries' pool, which they do without where it cannot be had; made now, while nothing is being captured
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    uint64_t keep = kPoolKeepBytes;
+    if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess) c->pool = nullptr;
+    else cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    cudaGetLastError();
     // the allocation-free entry point's array: loaded and located now, while allocating is allowed
     unsigned char *scratch = nullptr;
     if (noalloc_scratch(c, &scratch) != KNS_OK) {  // retried by the first kns_render_noalloc
@@ -1661,18 +1670,12 @@ static cudaError_t points_grouped(kns_ctx *ctx, const kns_grid *grid, const floa
                                   float *feat, float *grad, cudaStream_t s, bool &grouped) {
     const kns::GridView &g = grid->view;
     grouped = false;
-    if (!ctx->pool) {
-        cudaMemPoolProps props{};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = ctx->device;
-        if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess) {
-            ctx->pool = nullptr;
-            cudaGetLastError();
-            return cudaSuccess;
-        }
-        uint64_t keep = kPoolKeepBytes;
-        cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    // A call that is being captured goes point by point: scratch of a captured call belongs to its graph, and a graph
+    // with memory of its own can be instantiated only once at a time and be no part of another.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (!ctx->pool || cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return cudaSuccess;
     }
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t b_ctl = up(sizeof(int) * (2 + (size_t)g.ncl)), b_rank = up(sizeof(int) * (size_t)n),
