@@ -3,14 +3,14 @@
 // kns:instantiate (compiled once per grid configuration)
 //
 // A warp takes a tile of up to P points of one cell and runs the MLP forward, and backward from the d row
-// (as kns_shade.cu, in place), with the weights read from the cell's shading layout in global memory
+// (in place), with the weights read from the cell's shading layout in global memory
 // (kns_warp.cuh): 85 KB per tile at width 64, so what bounds a large batch is the latency and the number of
 // those reads.  Batches of a few points per cell and more are therefore grouped first -- a count per cell, a
 // segment per non-empty cell (segments in any order, so no scan across blocks), a scatter of (point, id) --
 // and evaluated in tiles of 16 points, each tile's weights on their way to L2 while the warp's previous tile
 // runs.  Smaller batches take one point per warp, ungrouped: nothing is gained by grouping when the cells
 // hold about one point each.  A thread per point, each reading its own cell's weights, was what this
-// replaced: 1,000,003 random points of 32^3 cells of width 64 took 52 ms, now 2.4 ms (2.9 GB of weights
+// replaced: 1,000,003 random points of 32^3 cells of width 64 took 52 ms, now 2.0 ms (2.9 GB of weights
 // once from memory: 0.43 ms at 6.8 TB/s; 12 warps per SM, 75 % of their time waiting for weight rows); 4,096
 // points of 16^3 cells of width 32 took 115 us, now 22 us (one wave of warps).
 #include <algorithm>
@@ -24,25 +24,39 @@ namespace {
 
 constexpr int PWARPS = 4;  // warps per block
 
-// shared rows of a warp: the encoding, A_1 .. A_H, and rows for W_0^T D_1 beyond those of A_2 .. A_H
+// softplus_beta'(s) = sigmoid(beta s), from the exponential softplus_f32 takes
+__device__ __forceinline__ float dsoftplus(float s, float beta) {
+    const float e = __expf(-beta * fabsf(s)), r = __fdividef(1.f, 1.f + e);
+    return s < 0.f ? e * r : r;
+}
+
+// shared rows of a warp: the encoding, A_1 .. A_H, and rows for W_0^T D_1 beyond those of A_2 .. A_H.  The gradient takes
+// softplus' from the sums, not from the activations as shading does: softplus_f32 rounds to zero where softplus' is below
+// 6e-8.  Either they lie in the layer's own rows, and its activations in the rows of the next layer (the last one's in its
+// own): `shifted`; or, for one point of width 32, a lane keeps its units' in registers.  (One point is bound by the
+// weight rows on their way, and so by how the compiler orders their loads: shifted, a query of width 32 for d alone
+// takes 17 us instead of 11 (64 points of a 16^3 grid); in registers, one of width 64 takes 52 us instead of 38.)
 template <class C>
 struct PL {
-    static constexpr int E = 0;
     __host__ __device__ static constexpr int A(int l) { return C::INP + (l - 1) * C::W; }
+    __host__ __device__ static constexpr int act(int l, bool shifted) { return shifted && l < C::H ? A(l + 1) : A(l); }
     static constexpr int G = C::INP + C::W;  // W_0^T D_1 over A_2 .. A_H, dead by then
     static constexpr int R0 = SL<C>::R0;
     static constexpr int ROWS = G + ((C::H - 1) * C::W > R0 ? (C::H - 1) * C::W : R0);
 };
 
 // The tile's points are in lanes 0 .. P - 1 (px, py, pz; id < 0: padding); M maps layers of width W to the
-// lanes, ME the encoding's gradient.
-template <class C, class M, class ME>
+// lanes, ME the encoding's gradient; GRAD: with the gradient, where the caller wants it (in a tile always; a branch between
+// its layers would keep the next layer's first weight rows from being loaded ahead of it).
+template <class C, class M, class ME, bool GRAD>
 __device__ __forceinline__ void points_tile(const GridView &g, const float *__restrict__ cw, float *rows, int lane,
                                             float px, float py, float pz, int64_t id, float *sdf, float *feat,
                                             float *grad) {
     using L = SL<C>;
     using R = PL<C>;
     constexpr int P = M::P, RS = row_stride(P), W = C::W;
+    constexpr bool SHIFT = GRAD && (P > 1 || W == 64);
+    float slope[C::H][P == 1 ? M::NU : 1];  // one point: softplus' of the lane's units
     if (lane < P) {  // Eq. 1, one lane per point
         float in[C::INP];
         encode3<C::L>(px, py, pz, in);
@@ -53,15 +67,22 @@ __device__ __forceinline__ void points_tile(const GridView &g, const float *__re
     M m(lane);
     m.fetch(cw + L::T0, W);
     auto act = [&](float v, int, int) { return softplus_f32(v, g.beta, g.inv_beta); };
+    auto dact = [&](float v, int, int) { return dsoftplus(v, g.beta); };
     m.bias(cw + L::b0);
     m.template mm<C::INP>(cw + L::T0, W, rows, RS, cw + L::Tl(1), W);
-    m.store(rows + R::A(1) * RS, RS, act);
+    m.store(rows + R::act(1, SHIFT) * RS, RS, act);
+    if constexpr (SHIFT) m.store(rows + R::A(1) * RS, RS, dact);
+    if constexpr (P == 1) m.each([&](float v, int i) { slope[0][i] = dsoftplus(v, g.beta); });
     __syncwarp();
 #pragma unroll
-    for (int l = 1; l < C::H; ++l) {
-        m.bias(cw + L::bl(l));
-        m.template mm<W>(cw + L::Tl(l), W, rows + R::A(l) * RS, RS, l + 1 < C::H ? cw + L::Tl(l + 1) : cw + L::Wlr(C::H - 1), W);
-        m.store(rows + R::A(l + 1) * RS, RS, act);
+    for (int l = 2; l <= C::H; ++l) {
+        m.bias(cw + L::bl(l - 1));
+        m.template mm<W>(cw + L::Tl(l - 1), W, rows + R::act(l - 1, SHIFT) * RS, RS,
+                         l < C::H ? cw + L::Tl(l) : cw + L::Wlr(C::H - 1), W);
+        if constexpr (SHIFT) __syncwarp();  // every lane has read the input, whose rows are written next
+        m.store(rows + R::act(l, SHIFT) * RS, RS, act);
+        if (SHIFT && l < C::H) m.store(rows + R::A(l) * RS, RS, dact);
+        if constexpr (P == 1) m.each([&](float v, int i) { slope[l - 1][i] = dsoftplus(v, g.beta); });
         __syncwarp();
     }
     if (feat) {  // the 16 outputs [d, z]: lane l < 16 output l of the first half of the points, lane l + 16 of the second
@@ -98,18 +119,22 @@ __device__ __forceinline__ void points_tile(const GridView &g, const float *__re
         sdf[id] = d;
     }
     __syncwarp();
-    if (!grad) return;
-    for (int i = lane; i < W * P; i += 32) {  // D_H = w_d . softplus'(A_H), in place
-        float *p = rows + (R::A(C::H) + i / P) * RS + i % P;
-        *p = __ldg(cw + L::wd + i / P) * dsoftplus_from_act(*p, g.beta);
-    }
+    if (!GRAD || !grad) return;
+    // D_H = w_d . softplus', over A_H
+    m.store(rows + R::A(C::H) * RS, RS, [&](float v, int u, int) {
+        if constexpr (P == 1 && !SHIFT) return __ldg(cw + L::wd + u) * slope[C::H - 1][u - m.u0];
+        else return __ldg(cw + L::wd + u) * dsoftplus(v, g.beta);
+    });
     __syncwarp();
 #pragma unroll
-    for (int l = C::H - 1; l >= 1; --l) {  // D_l = (W_l^T D_{l+1}) . softplus'(A_l) over A_l
+    for (int l = C::H - 1; l >= 1; --l) {  // D_l = (W_l^T D_{l+1}) . softplus', over the latter
         m.zero();
         m.template mm<W>(cw + L::Wlr(l), W, rows + R::A(l + 1) * RS, RS, l > 1 ? cw + L::Wlr(l - 1) : nullptr, W);
         float *own = rows + R::A(l) * RS;
-        m.store(own, RS, [&](float v, int u, int s) { return v * dsoftplus_from_act(own[u * RS + s], g.beta); });
+        m.store(own, RS, [&](float v, int u, int s) {
+            if constexpr (P == 1 && !SHIFT) return v * slope[l - 1][u - m.u0];
+            else return v * own[u * RS + s];
+        });
         __syncwarp();
     }
     ME e(lane);
@@ -139,7 +164,7 @@ __device__ __forceinline__ void points_tile(const GridView &g, const float *__re
 }
 
 // One point per warp, in the order given.
-template <class C>
+template <class C, bool GRAD>
 __global__ void __launch_bounds__(32 * PWARPS) points_direct_kernel(GridView g, const float *__restrict__ pts, int64_t n,
                                                                      float *sdf, float *feat, float *grad) {
     extern __shared__ __align__(16) float psm[];
@@ -150,13 +175,14 @@ __global__ void __launch_bounds__(32 * PWARPS) points_direct_kernel(GridView g, 
     if (q >= n) return;
     const float x = __ldg(pts + 3 * q), y = __ldg(pts + 3 * q + 1), z = __ldg(pts + 3 * q + 2);
     const int cell = cell_of(g, x, y, z);
-    points_tile<C, UnitMap<C::W>, UnitMap<PL<C>::R0>>(g, g.ws + (int64_t)cell * g.ws_stride, rows, lane, x, y, z,
-                                                      lane == 0 ? q : -1, sdf, feat, grad);
+    points_tile<C, UnitMap<C::W>, UnitMap<PL<C>::R0>, GRAD>(g, g.ws + (int64_t)cell * g.ws_stride, rows, lane, x, y, z,
+                                                            lane == 0 ? q : -1, sdf, feat, grad);
 }
 
-template <class C, int P>
-__global__ void __launch_bounds__(32 * PWARPS) points_tile_kernel(GridView g, PointsScratch s, float *sdf, float *feat,
-                                                                   float *grad) {
+// registers for as many blocks per SM as shared memory holds
+template <class C, int P, bool GRAD>
+__global__ void __launch_bounds__(32 * PWARPS, C::W == 32 ? 5 : 3) points_tile_kernel(GridView g, PointsScratch s, float *sdf,
+                                                                                      float *feat, float *grad) {
     extern __shared__ __align__(16) float psm[];
     constexpr int RS = row_stride(P);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -167,7 +193,7 @@ __global__ void __launch_bounds__(32 * PWARPS) points_tile_kernel(GridView g, Po
         const int tn = t + gridDim.x * PWARPS;  // the next tile's weights start for L2 while this one runs
         if (lane == 0 && tn < n_tiles) {
             const int c = s.tiles[tn].x;
-            prefetch_l2(g.ws + (int64_t)c * g.ws_stride, (grad ? SL<C>::C0t : SL<C>::W0r) * (int)sizeof(float));
+            prefetch_l2(g.ws + (int64_t)c * g.ws_stride, (GRAD ? SL<C>::C0t : SL<C>::W0r) * (int)sizeof(float));
         }
         float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
         int64_t id = -1;
@@ -175,22 +201,22 @@ __global__ void __launch_bounds__(32 * PWARPS) points_tile_kernel(GridView g, Po
             p = s.sorted[d.y + lane];
             id = __float_as_int(p.w);
         }
-        points_tile<C, TileMap<C::W, P>, TileMap<PL<C>::R0, P>>(g, g.ws + (int64_t)d.x * g.ws_stride, rows, lane, p.x, p.y,
-                                                            p.z, id, sdf, feat, grad);
+        points_tile<C, TileMap<C::W, P>, TileMap<PL<C>::R0, P>, GRAD>(g, g.ws + (int64_t)d.x * g.ws_stride, rows, lane, p.x,
+                                                                      p.y, p.z, id, sdf, feat, grad);
     }
 }
 
-template <class C, int P>
+template <class C, int P, bool GRAD>
 cudaError_t launch_tiles(const GridView &g, const PointsScratch &sc, int64_t n, float *sdf, float *feat, float *grad,
                          int sm_count, cudaStream_t s) {
     constexpr int smem = PWARPS * PL<C>::ROWS * row_stride(P) * (int)sizeof(float);
     static_assert(smem <= 200 * 1024, "point tiles do not fit in shared memory");
     static PerDevice per_sm;
     int nb = 0;
-    cudaError_t e = resident_blocks(points_tile_kernel<C, P>, 32 * PWARPS, smem, per_sm, nb);
+    cudaError_t e = resident_blocks(points_tile_kernel<C, P, GRAD>, 32 * PWARPS, smem, per_sm, nb);
     if (e != cudaSuccess) return e;
     const int64_t most = (n / P + g.ncl + PWARPS) / PWARPS;  // blocks that could have a tile
-    points_tile_kernel<C, P><<<(unsigned)std::min<int64_t>((int64_t)sm_count * nb, most), 32 * PWARPS, smem, s>>>(
+    points_tile_kernel<C, P, GRAD><<<(unsigned)std::min<int64_t>((int64_t)sm_count * nb, most), 32 * PWARPS, smem, s>>>(
         g, sc, sdf, feat, grad);
     return cudaGetLastError();
 }
@@ -201,16 +227,19 @@ template <class C>
 cudaError_t launch_points_direct_cfg(const GridView &g, const float *pts, int64_t n, float *sdf, float *feat,
                                      float *grad, cudaStream_t s) {
     constexpr int smem = PWARPS * PL<C>::ROWS * row_stride(1) * (int)sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(points_direct_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // width 32 has one kernel for both (compiled for d alone, it has fewer loads under way)
+    auto kernel = grad || C::W == 32 ? points_direct_kernel<C, true> : points_direct_kernel<C, C::W == 32>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    points_direct_kernel<C><<<(unsigned)((n + PWARPS - 1) / PWARPS), 32 * PWARPS, smem, s>>>(g, pts, n, sdf, feat, grad);
+    kernel<<<(unsigned)((n + PWARPS - 1) / PWARPS), 32 * PWARPS, smem, s>>>(g, pts, n, sdf, feat, grad);
     return cudaGetLastError();
 }
 
 template <class C>
 cudaError_t launch_points_tiles_cfg(const GridView &g, const PointsScratch &sc, int64_t n, float *sdf, float *feat,
                                     float *grad, int sm_count, cudaStream_t s) {
-    return launch_tiles<C, kPointsTile>(g, sc, n, sdf, feat, grad, sm_count, s);
+    return grad ? launch_tiles<C, kPointsTile, true>(g, sc, n, sdf, feat, grad, sm_count, s)
+                : launch_tiles<C, kPointsTile, false>(g, sc, n, sdf, feat, grad, sm_count, s);
 }
 
 #ifdef KNS_W

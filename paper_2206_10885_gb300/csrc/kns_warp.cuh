@@ -243,6 +243,12 @@ struct UnitMap {
 #pragma unroll
         for (int u = 0; u < NU; ++u) rows[(u0 + u) * xs] = f(acc[u], u0 + u, 0);
     }
+    // f(sum, index) of the lane's units
+    template <class F>
+    __device__ __forceinline__ void each(F f) const {
+#pragma unroll
+        for (int u = 0; u < NU; ++u) f(acc[u], u);
+    }
 };
 
 // Starts bringing `bytes` (a multiple of 16) at p (16-byte aligned) into L2.
