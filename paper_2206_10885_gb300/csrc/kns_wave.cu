@@ -482,6 +482,18 @@ struct EB {
     static constexpr int SMEM = (C::TSIZE + NW * ROWS * RS) * 4;
 };
 
+// A warp's wait for the tile's weights.  Where it runs out: reports, raises *fail and gives the copy once more the time to
+// land before the block's memory is another's.
+__device__ __forceinline__ bool weights_landed(uint64_t *bar, uint32_t phase, int lane, int *fail, int *status) {
+    if (__all_sync(FULL, mbar_wait(bar, phase, 1u << 26))) return true;
+    if (lane == 0) {
+        atomicCAS(status, 0, (int)6 /* KNS_ERR_TIMEOUT */);
+        *fail = 1;
+    }
+    mbar_wait(bar, phase, 1u << 26);
+    return false;
+}
+
 template <class C, bool STACK>
 __global__ void __launch_bounds__(EB<C>::NT, EB<C>::BLOCKS) wave_eval_warps_kernel(GridView g, WaveArgs a, int cur) {
     using B = EB<C>;
@@ -489,7 +501,7 @@ __global__ void __launch_bounds__(EB<C>::NT, EB<C>::BLOCKS) wave_eval_warps_kern
     extern __shared__ __align__(128) float dyn[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ int s_tile[2][4];  // cell, start, len, fresh; alternating
-    __shared__ int s_fail;
+    __shared__ int s_fail[2];     // a warp's wait for the tile's weights ran out; alternating
     if (a.ctrl->tail) return;  // finished one warp per ray by wave_tail_warp_kernel
     const int n_tiles = a.ctrl->n_tiles_fine;
     if (n_tiles <= 0) return;
@@ -497,7 +509,7 @@ __global__ void __launch_bounds__(EB<C>::NT, EB<C>::BLOCKS) wave_eval_warps_kern
     float *wsm = dyn, *A = dyn + C::TSIZE + warp * B::ROWS * RS;
     if (tid == 0) {
         mbar_init(&bar, 1);
-        s_fail = 0;
+        s_fail[0] = s_fail[1] = 0;
     }
     const int per = (n_tiles + gridDim.x - 1) / gridDim.x;
     int next_static = blockIdx.x * per;
@@ -524,7 +536,7 @@ __global__ void __launch_bounds__(EB<C>::NT, EB<C>::BLOCKS) wave_eval_warps_kern
         __syncthreads();  // and every warp is done with the previous tile's weights
         const int c = s_tile[par][0], start = s_tile[par][1], len = s_tile[par][2];
         bool wait = s_tile[par][3] != 0;
-        if (c < 0 || s_fail) break;
+        if (c < 0 || s_fail[par ^ 1]) break;  // (nothing sets the previous tile's flag any more: the block leaves together)
         cached = c;
         if (tid == 0) {
             if (wait) bulk_load(wsm, a.wt + (int64_t)c * a.wt_stride, C::TSIZE * sizeof(float), &bar);
@@ -574,13 +586,7 @@ __global__ void __launch_bounds__(EB<C>::NT, EB<C>::BLOCKS) wave_eval_warps_kern
             }
             if (wait) {
                 wait = false;
-                if (!__all_sync(FULL, mbar_wait(&bar, phase, 1u << 26))) {  // the weights never landed: report
-                    if (lane == 0) {
-                        atomicCAS(a.status, 0, (int)6 /* KNS_ERR_TIMEOUT */);
-                        s_fail = 1;
-                    }
-                    break;
-                }
+                if (!weights_landed(&bar, phase, lane, s_fail + par, a.status)) break;
                 phase ^= 1u;
             }
             __syncwarp();
@@ -664,7 +670,7 @@ __global__ void __launch_bounds__(EB<C>::NT, EB<C>::BLOCKS) wave_eval_warps_kern
             active = stay;
         }
         if (wait) {  // a warp without samples follows the weights' phase
-            if (!mbar_wait(&bar, phase, 1u << 26)) s_fail = 1;
+            weights_landed(&bar, phase, lane, s_fail + par, a.status);
             phase ^= 1u;
         }
     }
