@@ -87,6 +87,17 @@ def workload_config(name, desc, cams, W, H, ms, eps, precision):
                       "N(0, 1e-3) perturbation, seeded orbit cameras"}
 
 
+def fp32_launches(live, n_rays, n_cells, tail_rays):
+    """Kernels of one FP32 render whose rounds held `live` samples: ray generation, per round the scan (two launches
+    where there are more cells than one block takes), the scatter, the evaluation and the tail, between rounds the
+    walk of the rays waiting in empty voxels, then the hit sort (3) and shading.  The last round is evaluated by the
+    tail alone where the host knew that it would be: the whole render, or the round before, held no more rays than the
+    tail takes (it then counted the rays still waiting, which the trace does not tell: one launch at most is missed)."""
+    before = live[-2] if len(live) > 1 else n_rays
+    per_round = (2 if n_cells > 4096 else 1) + 3
+    return 1 + len(live) * per_round + len(live) - 1 + 4 - (1 if before <= tail_rays else 0)
+
+
 def mac_counts(desc):
     """Algorithmic multiply-adds: per trace sample (d only) and per hit (full SDF + gradient + colour)."""
     IN = 3 + 6 * desc.pe_pos_L
@@ -501,10 +512,12 @@ def run_kns(args, rank, world, local_rank):
                           "cooperative launch), the one-warp-per-ray tail, hit count/scan/scatter, shading, FP32 "
                           "refinement")
         else:
-            launches = 3 + st["rounds"] * 5
-            launch_src = ("library round counter, the fewest launches it stands for: gen + rounds x (scan, scatter, "
-                          "eval, tail) + (rounds - 1) advance + hit sort (3) + shade, less the evaluation of a last "
-                          "round that is the tail's (a scan of more than 4096 keys takes two launches, not counted)")
+            from paper_2206_10885_gb300 import autotune
+            tail = (tuning or autotune.default_setting(precision, desc.sdf_width))["tail_rays"]
+            launches = fp32_launches([r["live"] for r in trace], n_rays, desc.n_cells, tail)
+            launch_src = ("the rounds of the library's round trace: gen + per round a scan (two launches for more than "
+                          "4096 cells), scatter, evaluation and tail + (rounds - 1) advance + hit sort (3) + shade, "
+                          "less the evaluation of a last round that is the tail's")
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": max(3, args.warmup), "ms_per_step": ms_per_step, "higher_is_better": True,
                 "scaling": "weak", "vs_baseline": None, "dtype": "f32" if precision == kns.KNS_FP32 else "bf16",
