@@ -138,6 +138,12 @@ __device__ __forceinline__ float softplus_f32(float s, float beta, float inv_bet
 __device__ __forceinline__ float dsoftplus_f32(float s, float beta) {
     return 1.f / (1.f + __expf(-beta * s));
 }
+// the same from softplus_beta(s) = a: 1 - exp(-beta a), by its series for small a (shading and training keep activations
+// only; below 6e-8, where softplus_f32 rounds to zero, it is zero)
+__device__ __forceinline__ float dsoftplus_from_act(float a, float beta) {
+    const float x = beta * a;
+    return x < 1e-2f ? x * (1.f - x * (0.5f - x * (1.f / 6.f))) : 1.f - __expf(-x);
+}
 __device__ __forceinline__ float sigmoid_f32(float s) { return 1.f / (1.f + __expf(-s)); }
 
 // ------------------------------------------------------------------ Eq. 1 encoding

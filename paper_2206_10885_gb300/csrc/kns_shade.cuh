@@ -29,9 +29,4 @@ struct SL {
     static constexpr int Ud = R0 + C::H * W, U = Ud + 1, Hc = U + C::CINP, ROWS = Hc + W;
 };
 
-__device__ __forceinline__ float dsoftplus_from_act(float a, float beta) {
-    const float x = beta * a;  // sigmoid(beta s) = 1 - exp(-beta softplus_beta(s)); series for small x
-    return x < 1e-2f ? x * (1.f - x * (0.5f - x * (1.f / 6.f))) : 1.f - __expf(-x);
-}
-
 }  // namespace kns

@@ -48,17 +48,6 @@ struct WL {
     static constexpr int cc0 = cC0 + 33 * 32, cC1 = cc0 + 32, cc1 = cC1 + 96;
 };
 
-// ------------------------------------------------------------------ activations
-__device__ __forceinline__ float softplus(float s, float beta, float inv_beta) {
-    return fmaxf(s, 0.f) + __logf(1.f + __expf(-beta * fabsf(s))) * inv_beta;
-}
-// softplus_beta'(s) = sigmoid(beta s) = 1 - exp(-beta a) with a = softplus_beta(s) (series for small a)
-__device__ __forceinline__ float dsoftplus_act(float a, float beta) {
-    const float x = beta * a;
-    return x < 1e-2f ? x * (1.f - x * (0.5f - x * (1.f / 6.f))) : 1.f - __expf(-x);
-}
-__device__ __forceinline__ float sigm(float s) { return 1.f / (1.f + __expf(-s)); }
-
 // ------------------------------------------------------------------ records on warps
 // The kernels of the difference points and coarse samples (151 M records in a step of 2^18 rays) work on warp
 // tiles: a warp takes 32 records of the chunk's cell through every layer on its own rows in shared memory
@@ -123,7 +112,7 @@ __global__ void __launch_bounds__(32 * FW, FB) k_warp_eval_d(TrainArgs a, int k0
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float *rows = sw + S::FEND + warp * 32 * WRS;  // a layer overwrites its input
     const int c0 = a.chunk_off[k0], total = a.chunk_off[k1] - c0;
-    auto act = [&](float v, int, int) { return softplus(v, a.beta, a.inv_beta); };
+    auto act = [&](float v, int, int) { return softplus_f32(v, a.beta, a.inv_beta); };
     for (int ci = blockIdx.x; ci < total; ci += gridDim.x) {
         const int key = chunk_key(a.chunk_off, k0, k1, c0 + ci);
         const int j = c0 + ci - a.chunk_off[key];
@@ -227,7 +216,7 @@ __global__ void __launch_bounds__(32 * BW, 2) k_warp_fd_backward(TrainArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float *all = sw + S::END, *rows = all + warp * R::ROWS * WRS, *gr = rows + R::G * WRS;
     const int c0 = a.chunk_off[0], total = a.chunk_off[a.NC] - c0;
-    auto act = [&](float v, int, int) { return softplus(v, a.beta, a.inv_beta); };
+    auto act = [&](float v, int, int) { return softplus_f32(v, a.beta, a.inv_beta); };
     for (int ci = blockIdx.x; ci < total; ci += gridDim.x) {
         const int cell = chunk_key(a.chunk_off, 0, a.NC, c0 + ci);
         const int j = c0 + ci - a.chunk_off[cell];
@@ -277,7 +266,7 @@ __global__ void __launch_bounds__(32 * BW, 2) k_warp_fd_backward(TrainArgs a) {
                 float *own = rows + R::A(H) * WRS;
                 m.zero();
                 m.store(own, WRS, [&](float, int u, int s) {
-                    return sw[S::wo + u] * gr[s] * dsoftplus_act(own[u * WRS + s], a.beta);
+                    return sw[S::wo + u] * gr[s] * dsoftplus_from_act(own[u * WRS + s], a.beta);
                 });
             }
             __syncwarp();
@@ -290,7 +279,7 @@ __global__ void __launch_bounds__(32 * BW, 2) k_warp_fd_backward(TrainArgs a) {
                 m.zero();
                 m.template mm_shared<32>(sw + S::R(l), 32, D, WRS);
                 __syncwarp();  // A_l has been read
-                m.store(own, WRS, [&](float v, int u, int s) { return v * dsoftplus_act(own[u * WRS + s], a.beta); });
+                m.store(own, WRS, [&](float v, int u, int s) { return v * dsoftplus_from_act(own[u * WRS + s], a.beta); });
                 __syncwarp();
             }
             grad_tile32(rows + R::A(1) * WRS, rows, dw[0], lane);
@@ -416,7 +405,7 @@ __device__ __forceinline__ void centre_tile(const TrainArgs &a, const float *sw,
         }
     }
     __syncwarp();
-    auto act = [&](float v, int, int) { return softplus(v, a.beta, a.inv_beta); };
+    auto act = [&](float v, int, int) { return softplus_f32(v, a.beta, a.inv_beta); };
     TileMap<32, CT> m(lane);
 #pragma unroll
     for (int l = 0; l < H; ++l) {
@@ -500,9 +489,9 @@ __global__ void __launch_bounds__(32 * CFW, 2) k_warp_centre_fwd(TrainArgs a) {
             centre_tile<H, false>(a, sw, rows, lane, r, q, lg, gn);
             if (lane < 16 && q >= 0) {
                 a.d_c[q] = rows[R::Ud * CRS + lane];
-                a.rgb_c[3 * q] = sigm(lg[0]);
-                a.rgb_c[3 * q + 1] = sigm(lg[1]);
-                a.rgb_c[3 * q + 2] = sigm(lg[2]);
+                a.rgb_c[3 * q] = sigmoid_f32(lg[0]);
+                a.rgb_c[3 * q + 1] = sigmoid_f32(lg[1]);
+                a.rgb_c[3 * q + 2] = sigmoid_f32(lg[2]);
             }
             __syncwarp();
         }
@@ -596,7 +585,7 @@ __global__ void __launch_bounds__(32 * CBW, 1) k_warp_centre_backward(TrainArgs 
             if (lane < 16) {  // logits -> colour delta; the upstream of d
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    const float rgb = sigm(lg[c]);
+                    const float rgb = sigmoid_f32(lg[c]);
                     const float dc = up[c] * rgb * (1.f - rgb);
                     rows[(R::Dc + c) * CRS + lane] = dc;
                     dbc1[c] += dc;
@@ -650,7 +639,7 @@ __global__ void __launch_bounds__(32 * CBW, 1) k_warp_centre_backward(TrainArgs 
                 m.zero();
                 m.template mm_shared<16>(sw + S::Wo, 32, rows + R::Dout * CRS, CRS);
                 __syncwarp();
-                m.store(own, CRS, [&](float v, int u, int s) { return v * dsoftplus_act(own[u * CRS + s], a.beta); });
+                m.store(own, CRS, [&](float v, int u, int s) { return v * dsoftplus_from_act(own[u * CRS + s], a.beta); });
             }
             __syncwarp();
 #pragma unroll
@@ -662,7 +651,7 @@ __global__ void __launch_bounds__(32 * CBW, 1) k_warp_centre_backward(TrainArgs 
                 m.zero();
                 m.template mm_shared<32>(sw + W::R(l), 32, D, CRS);
                 __syncwarp();
-                m.store(own, CRS, [&](float v, int u, int s) { return v * dsoftplus_act(own[u * CRS + s], a.beta); });
+                m.store(own, CRS, [&](float v, int u, int s) { return v * dsoftplus_from_act(own[u * CRS + s], a.beta); });
                 __syncwarp();
             }
             grad_tile16<8>(rows + R::A(1) * CRS, rows, dw[0], lane);

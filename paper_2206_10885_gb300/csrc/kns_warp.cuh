@@ -15,13 +15,13 @@
 
 namespace kns {
 
-template <int W_, int P_, int G_ = 4>
+template <int W_, int P_>
 struct TileMap {
     static constexpr int W = W_, P = P_, NU = W / 8, S = P / 4;
-    static_assert(W % 32 == 0 && (S == 2 || S % 4 == 0), "tile shape");
+    static_assert(W % 32 == 0 && S % 4 == 0, "tile shape");
     f32x2 acc[NU][S / 2];
     int u0, s0;  // first unit, first sample
-    __device__ __forceinline__ explicit TileMap(int lane) : u0(4 * (lane >> 2)), s0((S == 2 ? 2 : 4) * (lane & 3)) {}
+    __device__ __forceinline__ explicit TileMap(int lane) : u0(4 * (lane >> 2)), s0(4 * (lane & 3)) {}
     __host__ __device__ static constexpr int unit(int i) { return (i & 3) + 32 * (i >> 2); }    // of u0
     __host__ __device__ static constexpr int sample(int j) { return (j & 3) + 16 * (j >> 2); }  // of s0
     __device__ __forceinline__ void bias(const float *b) {
@@ -44,7 +44,7 @@ struct TileMap {
     // Weight rows are loaded two groups of G inputs ahead of their products; fetch() loads the first two
     // groups of a matrix, which mm() finds loaded, and mm() in turn fetches those of `next` (so that they
     // arrive while the sums are finished and stored).
-    static constexpr int G = G_;
+    static constexpr int G = 4;
     float4 w[3][G * NU / 4];
     template <int B>
     __device__ __forceinline__ void fetch_to(const float *__restrict__ p, int ws) {
@@ -68,15 +68,11 @@ struct TileMap {
 #pragma unroll
         for (int k = 0; k < G; ++k) {
             f32x2 t[S / 2];
-            if constexpr (S == 2) {
-                t[0] = *reinterpret_cast<const f32x2 *>(x + k * xs);
-            } else {
 #pragma unroll
-                for (int j = 0; j < S / 4; ++j) {
-                    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(x + k * xs + 16 * j);
-                    t[2 * j] = v.x;
-                    t[2 * j + 1] = v.y;
-                }
+            for (int j = 0; j < S / 4; ++j) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(x + k * xs + 16 * j);
+                t[2 * j] = v.x;
+                t[2 * j + 1] = v.y;
             }
 #pragma unroll
             for (int h = 0; h < NU / 4; ++h) {
@@ -131,15 +127,11 @@ struct TileMap {
 #pragma unroll 4
         for (int k = 0; k < K; ++k) {
             f32x2 t[S / 2];
-            if constexpr (S == 2) {
-                t[0] = *reinterpret_cast<const f32x2 *>(xp + k * xs);
-            } else {
 #pragma unroll
-                for (int j = 0; j < S / 4; ++j) {
-                    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(xp + k * xs + 16 * j);
-                    t[2 * j] = v.x;
-                    t[2 * j + 1] = v.y;
-                }
+            for (int j = 0; j < S / 4; ++j) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(xp + k * xs + 16 * j);
+                t[2 * j] = v.x;
+                t[2 * j + 1] = v.y;
             }
 #pragma unroll
             for (int h = 0; h < NU / 4; ++h) {
@@ -171,20 +163,14 @@ struct TileMap {
 #pragma unroll
         for (int i = 0; i < NU; ++i) {
             const int u = u0 + unit(i);
-            if constexpr (S == 2) {
-                float a, b;
-                f2_unpack(acc[i][0], a, b);
-                *reinterpret_cast<float2 *>(rows + u * xs + s0) = make_float2(f(a, u, s0), f(b, u, s0 + 1));
-            } else {
 #pragma unroll
-                for (int j = 0; j < S; j += 4) {
-                    const int s = s0 + sample(j);
-                    float a, b, c, d;
-                    f2_unpack(acc[i][j / 2], a, b);
-                    f2_unpack(acc[i][j / 2 + 1], c, d);
-                    *reinterpret_cast<float4 *>(rows + u * xs + s) =
-                        make_float4(f(a, u, s), f(b, u, s + 1), f(c, u, s + 2), f(d, u, s + 3));
-                }
+            for (int j = 0; j < S; j += 4) {
+                const int s = s0 + sample(j);
+                float a, b, c, d;
+                f2_unpack(acc[i][j / 2], a, b);
+                f2_unpack(acc[i][j / 2 + 1], c, d);
+                *reinterpret_cast<float4 *>(rows + u * xs + s) =
+                    make_float4(f(a, u, s), f(b, u, s + 1), f(c, u, s + 2), f(d, u, s + 3));
             }
         }
     }
@@ -213,22 +199,13 @@ struct UnitMap {
     }
     __device__ __forceinline__ void fetch(const float *, int) {}
     template <int K>
-    __device__ __forceinline__ void mm(const float *__restrict__ w, int ws, const float *x, int xs, const float *, int) {
+    __device__ __forceinline__ void mm(const float *__restrict__ w, int ws, const float *x, int, const float *, int) {
         static_assert(K % 4 == 0, "layer input must be padded to 4");
         const float *wp = w + u0;
 #pragma unroll 4
         for (int k = 0; k < K; k += 4) {
-            float t[4];
-            if (xs == 1) {  // (a constant once inlined)
-                const float4 t4 = *reinterpret_cast<const float4 *>(x + k);
-                t[0] = t4.x;
-                t[1] = t4.y;
-                t[2] = t4.z;
-                t[3] = t4.w;
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) t[i] = x[(k + i) * xs];
-            }
+            const float4 t4 = *reinterpret_cast<const float4 *>(x + k);
+            const float t[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 float v[NU];
@@ -257,6 +234,6 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
 }
 
 // Row stride (floats) of P samples: the stores of a warp's units fall into distinct banks.
-__host__ __device__ constexpr int row_stride(int P) { return P == 1 ? 1 : P == 8 ? 10 : P + 4; }
+__host__ __device__ constexpr int row_stride(int P) { return P == 1 ? 1 : P + 4; }
 
 }  // namespace kns
