@@ -133,7 +133,10 @@ typedef struct kns_render_opts {
     int32_t inner_steps;   /* evaluations a tile may make per round while its rays stay in its cell (1..1024;
                               default 4 for warp tiles, 2 for block tiles) */
     int32_t min_active;    /* a tile continues only while at least this many of its rays stay in its cell
-                              (1..256; a warp tile holds 16; default 8 for warp tiles, 16 for block tiles) */
+                              (1..256; a warp tile holds 16; default 8 for warp tiles, 16 for block tiles).
+                              block_tiles 4: each warp decides for itself, and goes on while at least
+                              min_active / 128 of its samples, rounded down, and one stay (32 or, at SDF width
+                              64, 16 of them; more than 128: never) */
     int32_t tail_rays;     /* a round with at most this many rays is finished one warp per ray, in FP32 (>= 0;
                               -1: never; default: KNS_FP32 98304 at SDF width 32, 32768 at width 64; KNS_BF16
                               32768 at width 32, 16384 at width 64) */

@@ -422,16 +422,18 @@ kns_status with_room(kns_ctx *ctx, F f) {
 
 // Render tiling: samples per tile (a warp tile, or a 256-thread block tile).
 constexpr int kRenderBlockTile = 16;        // samples per warp tile
-constexpr int kRenderBlockTiles = 4;        // FP32 renders use 128-sample block tiles of 128 threads
+constexpr int kRenderBlockTiles = 4;        // FP32 renders use 128-sample block tiles split between warps
 // Defaults picked by the autotuner on the 16^3 / width-32 grid at 8 x 800x800.
 constexpr int kRenderInnerSteps = 4;
 constexpr int kRenderMinActive = 8;
 constexpr int kRenderBlockInnerSteps = 2;  // block tiles: a second evaluation of a tile in the round ...
-constexpr int kRenderBlockMinActive = 16;  // ... while at least 16 of its rays stay in its cell
+constexpr int kRenderBlockMinActive = 16;  // ... while at least 16 of its 128 rays (of each warp its share) stay in its cell
 // FP32 rounds this small finish one warp per ray (width 32).  The tail takes a sample every ~205 cycles of an SM (its
-// shared memory: weights read once per sample, copied for half of them), a light round ~110 us; of 8,192 .. 196,608
-// rays (65,536 / 98,304 / 131,072): eight 800 x 800 views 6.28 / 6.30 / 6.32 ms, five views of a stack of two grids
-// 2.00 / 1.99 / 2.03 ms, 100,003 rays 0.68 / 0.67 / 0.67 ms.
+// shared memory: weights read once per sample, copied for half of them), a light round ~110 us.  32,768 / 65,536 /
+// 98,304 / 131,072 rays, medians of ten passes taken in turn (quartiles 0.2 to 0.5 % apart): eight 800 x 800 views
+// 6.43 / 6.27 / 6.25 / 6.27 ms (other cameras 6.07 / 5.91 / 5.88 / 5.93), five views of a stack of two grids 2.18 /
+// 2.08 / 2.06 / 2.08 ms, 100,003 rays 0.90 / 0.70 / 0.70 / 0.69 ms, a path trace 1.42 / 1.20 / 1.20 / 1.20 ms: flat
+// from 65,536 on, 98,304 first or within a quartile of it everywhere.
 constexpr int kRenderTailRays = 98304;
 // Cells of all grids of a stack: the BF16 seam trap keeps a cell number in 19 bits.
 constexpr int64_t kMaxStackCells = 262144;

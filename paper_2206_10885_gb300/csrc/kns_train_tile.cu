@@ -14,7 +14,8 @@
 // x 96 samples and 16,384 eikonal points on a GB300: difference points forward 7.1 ms, centres forward 2.5,
 // centres backward 10.6, difference points backward 28.6 ms; now 6.3, 2.2, 7.1 and 18.8 ms (the step 51.2 -> 36.6
 // ms; 1,024 rays 3.0 -> 2.2 ms).  The forward kernel keeps the FP32 pipe 58 % busy; the backward ones have eight
-// warps of 255 registers per SM and wait on shared loads and instruction fetch: unrolling the weight-gradient
+// warps per SM (238 registers a thread for the difference points, 255 for the centres) and wait for the results of
+// their own FMA chains, on shared loads and on instruction fetch: unrolling the weight-gradient
 // loop twice costs 4.7 ms, five warps of 168 registers the same, loads a half step ahead 2.9 ms.
 //
 // Kernels: d at records (coarse samples and difference points); sample centres forward (d, z,
@@ -155,7 +156,7 @@ __global__ void __launch_bounds__(32 * FW, FB) k_warp_eval_d(TrainArgs a, int k0
 // of the whole chunk stay in registers -- lane (og, ig) = (lane / 8, lane % 8) owns outputs og + 4 i and inputs
 // ig + 8 j of every layer, 12 loads of 16 bytes for 128 FMAs -- and are summed over the block's warps in shared
 // memory and added to the global gradient once per chunk.
-constexpr int BW = 4;  // warps per block, two blocks per SM: 255 registers, 101 of them gradient sums
+constexpr int BW = 4;  // warps per block, two blocks per SM: 238 registers, 101 of them gradient sums
 template <int H>
 struct WRows {
     __host__ __device__ static constexpr int A(int l) { return 32 * l; }  // A(0): the encoding

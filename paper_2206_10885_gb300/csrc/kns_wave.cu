@@ -799,8 +799,8 @@ __device__ __forceinline__ float warp_d_row(const float *__restrict__ drow, floa
 // The weights of its cell that a lane of the tail keeps in registers: those of the last hidden layer, at width 32 with
 // three hidden layers.  The tail is bound by its SMs' shared memory -- 92 cycles of weight reads a sample there, 46 of inputs,
 // 32 of the d row and about 43 of the copies of the cells, one for every 2.3 samples -- and the register copy saves a
-// read of 32 cycles wherever the ray stays in its cell: eight 800 x 800 views 6.09 -> 6.02 ms, 100,003 rays 0.67 ->
-// 0.66 ms.  It costs 32 registers a lane, which are free only while the slots leave no more than 16 warps an SM: with
+// read of 32 cycles wherever the ray stays in its cell: eight 800 x 800 views 6.32 -> 6.24 ms, 100,003 rays 0.699 ->
+// 0.690 ms (medians of 22 passes, three processes of each in turn: no two of a side differ by more than 0.3 %).  It costs 32 registers a lane, which are free only while the slots leave no more than 16 warps an SM: with
 // two hidden layers the slots hold 24, the registers then 18 (four 64 x 64 views 0.181 -> 0.189 ms); two layers in
 // registers are slower (five views of a stack of two grids 2.01 -> 2.06 ms), and at width 64 one saves nothing.
 template <class C>
