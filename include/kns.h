@@ -359,7 +359,7 @@ kns_status kns_path_trace(kns_ctx *ctx, const kns_grid *grid, const kns_camera *
  * n x 3 FP32, row-major) evaluate the SDF MLP of cell m(x): sdf (device, n floats), feat (device,
  * n x feat_dim, or NULL), grad (device, n x 3 analytic input gradient, or NULL).
  * n = 0 is a successful no-op.  Queries of 32,768 points or more, four a cell on average, are grouped by cell
- * in stream-ordered scratch of the context's own pool (about 24 bytes a point, at most 128 MB kept between
+ * in stream-ordered scratch of the context's own pool (21 bytes a point and 36 a cell, at most 128 MB kept between
  * calls), or answered point by point where that cannot be allocated and where cuda_stream is being captured (so a
  * captured query is kernel launches alone).
  * Errors: INVALID_ARG (NULL pts/sdf with n > 0, n < 0), CUDA. */

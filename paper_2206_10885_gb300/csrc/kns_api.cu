@@ -451,10 +451,11 @@ constexpr int kRenderBlocksPerSM = 16;
 constexpr int kRenderStaticTiles = 2;
 
 // Field queries of at least this many points, and of at least this many per cell, are grouped by cell
-// (kns_points.cu); smaller ones take one point per warp.  Grouped / ungrouped, with feature and gradient, on
-// a GB300: 16^3 cells of width 32: 32,768 points 75 / 80 us, 65,536 points 82 / 147 us; 8^3 cells: 4,096
-// points 36 / 21 us, 32,768 points 45 / 46 us; 32^3 cells of width 64: 65,536 points (2 per cell)
-// 1.13 / 0.76 ms, 131,072 points 1.21 / 1.52 ms, 1,000,003 points 2.4 / 11.6 ms.
+// (kns_points.cu); smaller ones take one point per warp.  Grouped / ungrouped, uniform points, with feature and
+// gradient and the call's own 30 us, on a GB300: 16^3 cells of width 32: 16,384 points 113 / 88 us, 32,768 109 / 120,
+// 65,536 117 / 187; 8^3 cells: 16,384 points 72 / 61 us, 32,768 75 / 81; 32^3 cells of width 64: 65,536 points (2 per
+// cell) 0.95 / 0.81 ms, 131,072 1.08 / 1.56, 1,000,003 1.99 / 11.6.  Points near a surface fill few cells and would gain
+// from fewer on (100,000 of a sphere in 32^3 cells 0.21 / 0.50 ms), but how many they fill is known only once counted.
 constexpr int64_t kPointsGrouped = 32768, kPointsPerCellGrouped = 4;
 constexpr uint64_t kPoolKeepBytes = 128u << 20;  // scratch of field queries a context keeps between calls
 

@@ -11,8 +11,8 @@
 // runs.  Smaller batches take one point per warp, ungrouped: nothing is gained by grouping when the cells
 // hold about one point each.  A thread per point, each reading its own cell's weights, was what this
 // replaced: 1,000,003 random points of 32^3 cells of width 64 took 52 ms, now 2.0 ms (2.9 GB of weights
-// once from memory: 0.43 ms at 6.8 TB/s; 12 warps per SM, 75 % of their time waiting for weight rows); 4,096
-// points of 16^3 cells of width 32 took 115 us, now 22 us (one wave of warps).
+// once from memory: 0.43 ms at 6.8 TB/s; 12 warps per SM, 60 % of their time waiting for weight rows); 4,096
+// points of 16^3 cells of width 32 took 115 us, now 21 us (one wave of warps).
 #include <algorithm>
 
 #include "kns_shade.cuh"
